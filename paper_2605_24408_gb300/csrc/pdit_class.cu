@@ -113,14 +113,11 @@ __device__ __forceinline__ void run_class_replica(const SweepArgs &a, int r, int
             const int cnt = min(32, n - i0);
             for (int ii = 0; ii < cnt; ++ii) {
                 const int i = i0 + ii;
-                const unsigned long long draw =
-                    ((unsigned long long)__shfl_sync(kFull, rw.y, ii) << 32) |
-                    (unsigned long long)__shfl_sync(kFull, rw.x, ii);
+                const uint32_t draw_hi = __shfl_sync(kFull, rw.y, ii);
                 const int xa = sx[sp[i]];
                 const int gi = sG[i];
                 const DT *Di = sD + i * n;
                 // ---- swap energies: 0 within a class, 2 f (G_w - G_u - D_uw) across
-                int lmin = 0x7FFFFFFF;
                 int dself = 0;  // MAXK = 1: this thread's energy, handed to the draw in a register
 #pragma unroll
                 for (int k = 0; k < MAXK; ++k) {
@@ -135,10 +132,11 @@ __device__ __forceinline__ void run_class_replica(const SweepArgs &a, int r, int
                             sv[j] = d;
                         else
                             dself = d;
-                        lmin = min(lmin, d);
                     }
                 }
-                const int3 sel = eq5_draw<MAXK, WPR>(sv, sp, n, t, lmin, dself, MAXK == 1 && t < n ? sp[t] : 0, beta, draw, bar, gs);
+                const int3 sel = eq5_draw<MAXK, WPR>(
+                    sv, sp, n, t, dself, MAXK == 1 && t < n ? sp[t] : 0, beta, draw_hi,
+                    [&]() { return __shfl_sync(kFull, rw.x, ii); }, draw_tag(i, s), bar, gs);
                 const int js = sel.x, dstar = sel.y, fb = sel.z;
                 if (js == i) continue;
                 const int fa = sp[i];

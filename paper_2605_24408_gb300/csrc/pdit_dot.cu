@@ -199,7 +199,7 @@ __device__ __forceinline__ void run_dot_replica(const SweepArgs &a, int r, int t
         // `fix`, rowB and colB hold the entries of the next location i + 1
         // (computed from the same state) and are brought up to date when
         // the update swaps, before the rows of Q move.
-        auto step = [&](const int i, const unsigned long long draw, const int (&rowv)[MAXK],
+        auto step = [&](const int i, const int ii, const uint4 &rw, const int (&rowv)[MAXK],
                         const int (&colv)[MAXK], const bool fix, int (&rowB)[MAXK], int (&colB)[MAXK]) {
             const int si = dot_slot<MAXK>(i, TA);
             const int hi = sh[i];
@@ -208,7 +208,6 @@ __device__ __forceinline__ void run_dot_replica(const SweepArgs &a, int r, int t
 
             // ---- swap energies (Eq. 3 in the one-term units)
             int dc[MAXK];
-            int lmin = 0x7FFFFFFF;
 #pragma unroll
             for (int k = 0; k < MAXK; ++k) {
                 const int j = t * MAXK + k;
@@ -225,7 +224,6 @@ __device__ __forceinline__ void run_dot_replica(const SweepArgs &a, int r, int t
                     }
                     if (j == i) d = 0;
                     dc[k] = d;
-                    lmin = min(lmin, d);
                 }
             }
             auto fac = [&](int kk) {  // pc[kk] without indexing registers at run time
@@ -235,7 +233,9 @@ __device__ __forceinline__ void run_dot_replica(const SweepArgs &a, int r, int t
                     if (k == kk) v = pc[k];
                 return v;
             };
-            const int3 sel = eq5_draw_regs<MAXK, WPR>(dc, fac, n, t, lmin, beta_now, draw, bar, gs);
+            const int3 sel = eq5_draw_regs<MAXK, WPR>(
+                dc, fac, n, t, beta_now, __shfl_sync(kFull, rw.y, ii),
+                [&]() { return __shfl_sync(kFull, rw.x, ii); }, draw_tag(i, s), bar, gs);
             const int js = sel.x, dstar = sel.y, fb = sel.z;
             if (js == i) return;
 
@@ -426,16 +426,8 @@ __device__ __forceinline__ void run_dot_replica(const SweepArgs &a, int r, int t
                         }
                     }
                 }
-                const unsigned long long drawA =
-                    ((unsigned long long)__shfl_sync(kFull, rw.y, ii) << 32) |
-                    (unsigned long long)__shfl_sync(kFull, rw.x, ii);
-                step(i, drawA, rowA, colA, two, rowB, colB);
-                if (two) {
-                    const unsigned long long drawB =
-                        ((unsigned long long)__shfl_sync(kFull, rw.y, ii + 1) << 32) |
-                        (unsigned long long)__shfl_sync(kFull, rw.x, ii + 1);
-                    step(i + 1, drawB, rowB, colB, false, rowB, colB);
-                }
+                step(i, ii, rw, rowA, colA, two, rowB, colB);
+                if (two) step(i + 1, ii + 1, rw, rowB, colB, false, rowB, colB);
             }
         }
     }

@@ -269,23 +269,54 @@ __device__ __forceinline__ void fisher_yates(const SweepArgs &a, uint32_t grep, 
 
 // ---------------------------------------------------------------------------
 // Eq. 5 draw over n outcomes held thread-contiguously: thread t holds the
-// swap energies of outcomes t*MAXK + k (k < MAXK; outcomes >= n are ignored),
-// which `load(dc)` fills in once the group minimum is known (so energies that
-// other threads wrote to shared memory are read after the synchronisation of
-// the minimum), and `fac(k)` gives the facility at outcome t*MAXK + k (called
-// on the owning thread only); lmin is the minimum over this thread's own
-// outcomes. Group minimum, binary32 weights of the shifted energies, 64-bit
-// prefix sums in outcome order, the 64-bit draw scaled by the total, and the
-// first outcome whose inclusive prefix sum exceeds it. Returns (chosen
-// location js, its energy change, the facility at js), the same on every
-// thread of the group; the facility is read by the owning thread before the
-// final synchronisation. Ends with the group synchronised.
+// swap energies dc[k] of outcomes t*MAXK + k (k < MAXK; outcomes >= n are
+// ignored) and `fac(k)` gives the facility at outcome t*MAXK + k (called on
+// the owning thread only). The drawn outcome is defined by integers: weights
+// W_j = eq5_weight(dc_j - min) and the first j whose prefix sum P_j exceeds
+// floor(draw T / 2^64), T the total; equivalently, as P is integral, the j
+// with P_{j-1} <= U T < P_j, U = draw / 2^64.
+//
+// eq5_draw_exact computes just that. eq5_draw_core first draws with binary32
+// weights w_j = 2^(-beta log2(e) dc_j) (the stay outcome, dc = 0, is the
+// reference: no minimum is needed), their prefix sums and t = u total, and
+// keeps the outcome only if t - m and t + m, m = 2^-15 total, both fall
+// inside its interval; otherwise (and when total >= 2^64, infinite or not a
+// number) the exact draw decides. Both prefix distributions approximate that
+// of e^(-beta dc_j):
+//   exact: the argument's two roundings, <= 40 x 2^-23, the polynomial and
+//     its reduction, < 2^-20, the weights cut beyond 40 and the truncation,
+//     < 2^-40: relative 6e-6 a weight;
+//   binary32: arguments that matter lie in [-40, 64] (total < 2^64; terms
+//     below 2^-40 of the stay weight carry nothing) and have four roundings,
+//     64 x 3.5 x 2^-24 x ln 2 = 9.3e-6, and ex2.approx, 2^-22: 9.6e-6.
+// A prefix share F = A/(A+B) moves by F (1 - F) times the difference of the
+// relative errors, at most half of each bound, 7.8e-6 together; the binary32
+// sums add at most 20 roundings, 1.2e-6, twice, and u and t 2 x 2^-24. The
+// sum, 1.1e-5, is a third of 2^-15, so a kept outcome is the exact one. The
+// exact draw runs where t lies within m of a boundary: at most 2^-14 per
+// boundary that carries weight (0.6% of draws at n = 100 and beta = 0).
 // ---------------------------------------------------------------------------
-template <int MAXK, int WPR, typename Load, typename Fac>
-__device__ __forceinline__ int3 eq5_draw_core(Load load, Fac fac, int n, int t, int lmin, float beta,
-                                              unsigned long long draw, int bar, GroupScratch *gs) {
+constexpr float kDrawMargin = 3.0517578125e-05f;   // 2^-15
+constexpr float kDrawLimit = 1.8446744073709552e19f;  // 2^64
+constexpr float kLog2e = 1.44269502f;
+
+// 2^x, x in binary32 (error below 2^-22 relative; 0 for results below 2^-126).
+__device__ __forceinline__ float ex2_approx(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// The draw by 64-bit integer prefix sums. Ends with the group synchronised.
+template <int MAXK, int WPR, typename Fac>
+__device__ __forceinline__ int3 eq5_draw_exact(const int (&dc)[MAXK], Fac fac, int n, int t, float beta,
+                                               unsigned long long draw, int tag, int bar, GroupScratch *gs) {
     const int lane = t & 31;
     const int wg = t >> 5;
+    int lmin = 0x7FFFFFFF;
+#pragma unroll
+    for (int k = 0; k < MAXK; ++k)
+        if (t * MAXK + k < n) lmin = min(lmin, dc[k]);
     int dmin = __reduce_min_sync(kFull, lmin);
     if constexpr (WPR > 1) {
         if (lane == 0) gs->wmin[wg] = dmin;
@@ -293,13 +324,8 @@ __device__ __forceinline__ int3 eq5_draw_core(Load load, Fac fac, int n, int t, 
         dmin = gs->wmin[0];
 #pragma unroll
         for (int w = 1; w < WPR; ++w) dmin = min(dmin, gs->wmin[w]);
-    } else {
-        __syncwarp();
     }
 
-    // ---- sample: thread-contiguous weights, 64-bit prefix sums
-    int dc[MAXK];
-    load(dc);
     unsigned long long pre[MAXK];
     unsigned long long lsum = 0;
 #pragma unroll
@@ -346,33 +372,132 @@ __device__ __forceinline__ int3 eq5_draw_core(Load load, Fac fac, int n, int t, 
     }
     int js, dstar, fb;
     if constexpr (WPR > 1) {
-        // both below 2^16 (n <= 256): one 64-bit store and load
-        if (own) *reinterpret_cast<int2 *>(&gs->sel_jf) = make_int2(jloc | (fsel << 16), dsel);
+        // both below 2^8 (n <= 256)
+        if (own) *reinterpret_cast<int2 *>(&gs->sel_jf) = make_int2(jloc | (fsel << 8) | (tag << 16), dsel);
         group_sync<WPR>(bar);
         const int2 sel = *reinterpret_cast<const int2 *>(&gs->sel_jf);
-        js = sel.x & 0xFFFF;
-        fb = sel.x >> 16;
+        js = sel.x & 0xFF;
+        fb = (sel.x >> 8) & 0xFF;
         dstar = sel.y;
     } else {
         const int src = __ffs(__ballot_sync(kFull, own)) - 1;
         js = __shfl_sync(kFull, jloc, src);
         dstar = __shfl_sync(kFull, dsel, src);
         fb = __shfl_sync(kFull, fsel, src);
-        __syncwarp();
     }
     return make_int3(js, dstar, fb);
 }
 
+// The draw. Returns (chosen location js, its energy change, the facility at
+// js), the same on every thread of the group; the facility is read by the
+// owning thread before the last synchronisation. SYNC: the energies that
+// `load(dc)` reads come from other threads through shared memory, so the
+// group synchronises first. `draw_hi` is the high word of the 64-bit draw
+// and draw_lo() gives the low word (called where the exact draw runs). `tag`
+// is draw_tag: an outcome published under another tag is an old one, so no
+// thread kept its outcome and the exact draw runs. Ends with the group
+// synchronised.
+template <int MAXK, int WPR, bool SYNC, typename Load, typename Fac, typename Lo>
+__device__ __forceinline__ int3 eq5_draw_core(Load load, Fac fac, int n, int t, float beta, uint32_t draw_hi,
+                                              Lo draw_lo, int tag, int bar, GroupScratch *gs) {
+    const int lane = t & 31;
+    const int wg = t >> 5;
+    if constexpr (SYNC) group_sync<WPR>(bar);
+    int dc[MAXK];
+    load(dc);
+    const float kb = -beta * kLog2e;
+    float pre[MAXK];
+    float lsum = 0.0f;
+#pragma unroll
+    for (int k = 0; k < MAXK; ++k) {
+        const float w = ex2_approx(__int2float_rn(dc[k]) * kb);
+        lsum += t * MAXK + k < n ? w : 0.0f;
+        pre[k] = lsum;
+    }
+    float incl = lsum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+    }
+    float total;
+    if constexpr (WPR > 1) {
+        float *wt = reinterpret_cast<float *>(gs->wtot);
+        if (lane == 31) wt[wg] = incl;
+        group_sync<WPR>(bar);
+        float off = 0.0f;
+        total = 0.0f;
+#pragma unroll
+        for (int w = 0; w < WPR; ++w) {
+            const float v = wt[w];
+            off += w < wg ? v : 0.0f;
+            total += v;
+        }
+        incl += off;
+    } else {
+        total = __shfl_sync(kFull, incl, 31);
+    }
+    // (a total that is infinite or not a number makes every comparison fail)
+    const float u = __uint2float_rn(draw_hi >> 8) * 5.9604644775390625e-08f;
+    const float tt = u * total;
+    const float m = total < kDrawLimit ? kDrawMargin * total : __int_as_float(0x7FC00000);
+    const float tl = tt - m, th = tt + m;
+    const float excl = incl - lsum;
+    int kk = -1;
+    float lo = excl;
+#pragma unroll
+    for (int k = 0; k < MAXK; ++k) {
+        const float hi = excl + pre[k];
+        if (tl >= lo && th < hi) kk = k;
+        lo = hi;
+    }
+    const bool own = kk >= 0;
+    int jf = 0, dsel = 0;
+    if (own) {
+#pragma unroll
+        for (int k = 0; k < MAXK; ++k)
+            if (k == kk) dsel = dc[k];
+        jf = (t * MAXK + kk) | (fac(kk) << 8) | (tag << 16);
+    }
+    bool kept;
+    if constexpr (WPR > 1) {
+        if (own) *reinterpret_cast<int2 *>(&gs->sel_jf) = make_int2(jf, dsel);
+        group_sync<WPR>(bar);
+        const int2 sel = *reinterpret_cast<const int2 *>(&gs->sel_jf);
+        jf = sel.x;
+        dsel = sel.y;
+        kept = (int)((uint32_t)jf >> 16) == tag;
+    } else {
+        const unsigned b = __ballot_sync(kFull, own);
+        kept = b != 0;
+        const int src = __ffs(b) - 1;
+        jf = __shfl_sync(kFull, jf, src);
+        dsel = __shfl_sync(kFull, dsel, src);
+    }
+    if (!kept) {
+        const unsigned long long draw = ((unsigned long long)draw_hi << 32) | (unsigned long long)draw_lo();
+        return eq5_draw_exact<MAXK, WPR>(dc, fac, n, t, beta, draw, tag, bar, gs);
+    }
+    if constexpr (WPR == 1) __syncwarp();
+    return make_int3(jf & 0xFF, dsel, (jf >> 8) & 0xFF);
+}
+
+// Tag of the draw of location i in sweep s. Every draw leaves its tag in the
+// scratch, so the one a draw could meet there is its predecessor's, of
+// another location; the top bit keeps it apart from the work-unit numbers
+// that share the word.
+__device__ __forceinline__ int draw_tag(int i, int s) { return i | ((s & 0x7F) << 8) | 0x8000; }
+
 // The draw over energies that each thread holds in registers for its own
 // outcomes t*MAXK + k.
-template <int MAXK, int WPR, typename Fac>
-__device__ __forceinline__ int3 eq5_draw_regs(const int (&dc)[MAXK], Fac fac, int n, int t, int lmin, float beta,
-                                              unsigned long long draw, int bar, GroupScratch *gs) {
+template <int MAXK, int WPR, typename Fac, typename Lo>
+__device__ __forceinline__ int3 eq5_draw_regs(const int (&dc)[MAXK], Fac fac, int n, int t, float beta,
+                                              uint32_t draw_hi, Lo draw_lo, int tag, int bar, GroupScratch *gs) {
     auto load = [&](int (&o)[MAXK]) {
 #pragma unroll
         for (int k = 0; k < MAXK; ++k) o[k] = dc[k];
     };
-    return eq5_draw_core<MAXK, WPR>(load, fac, n, t, lmin, beta, draw, bar, gs);
+    return eq5_draw_core<MAXK, WPR, false>(load, fac, n, t, beta, draw_hi, draw_lo, tag, bar, gs);
 }
 
 // The draw over energies the group has written to sv[0..n) in location
@@ -380,10 +505,10 @@ __device__ __forceinline__ int3 eq5_draw_regs(const int (&dc)[MAXK], Fac fac, in
 // energy in dself and its location's facility in pself instead, and sv is
 // not read). The facility of the drawn location is read from sp by its
 // owner, so the caller may rewrite sp once every thread has returned.
-template <int MAXK, int WPR>
-__device__ __forceinline__ int3 eq5_draw(const int32_t *sv, const int32_t *sp, int n, int t, int lmin,
-                                         int dself, int pself, float beta, unsigned long long draw,
-                                         int bar, GroupScratch *gs) {
+template <int MAXK, int WPR, typename Lo>
+__device__ __forceinline__ int3 eq5_draw(const int32_t *sv, const int32_t *sp, int n, int t, int dself, int pself,
+                                         float beta, uint32_t draw_hi, Lo draw_lo, int tag, int bar,
+                                         GroupScratch *gs) {
     auto load = [&](int (&o)[MAXK]) {
         if constexpr (MAXK == 1)
             o[0] = dself;
@@ -391,7 +516,7 @@ __device__ __forceinline__ int3 eq5_draw(const int32_t *sv, const int32_t *sp, i
             load_block<MAXK>(sv, t, o);
     };
     auto fac = [&](int kk) { return MAXK == 1 ? pself : sp[t * MAXK + kk]; };
-    return eq5_draw_core<MAXK, WPR>(load, fac, n, t, lmin, beta, draw, bar, gs);
+    return eq5_draw_core<MAXK, WPR, (MAXK > 1)>(load, fac, n, t, beta, draw_hi, draw_lo, tag, bar, gs);
 }
 
 // Bytes of packed word w that hold one of the np pending terms (4 per word).
@@ -928,9 +1053,6 @@ __device__ __forceinline__ void run_replica(const SweepArgs &a, int part_arg, in
                 const int nrows = min(32, (n - ib + WPR - 1) / WPR);
                 for (int q = 0; q < nrows; ++q) {
                     const int i = ib + WPR * q;
-                    const unsigned long long draw =
-                        ((unsigned long long)__shfl_sync(kFull, rw.y, q) << 32) |
-                        (unsigned long long)__shfl_sync(kFull, rw.x, q);
                     const int fa = sp[i];
                     const int hi = sh[i];
                     const DT *Di = sD + i * dn;
@@ -944,7 +1066,6 @@ __device__ __forceinline__ void run_replica(const SweepArgs &a, int part_arg, in
                         }
                     }
                     int dv[ROWS];
-                    int lmin = 0x7FFFFFFF;
 #pragma unroll
                     for (int k = 0; k < ROWS; ++k) {
                         const int j = lane + 32 * k;
@@ -980,43 +1101,92 @@ __device__ __forceinline__ void run_replica(const SweepArgs &a, int part_arg, in
                                          ((int)Fa[fa] + (int)sF[b * n + b] - 2 * fab);
                             }
                             if (j == i) d = 0;
-                            lmin = min(lmin, d);
                         }
                         dv[k] = d;
                     }
-                    const int dmin = __reduce_min_sync(kFull, lmin);
-                    unsigned long long incl[ROWS], tot[ROWS];
+                    // binary32 draw, kept where it is certainly the exact
+                    // one (eq5_draw_core; outcome 32 k + lane, prefix sums
+                    // in that order)
+                    const uint32_t draw_hi = __shfl_sync(kFull, rw.y, q);
+                    const float kb = -beta * kLog2e;
+                    float wk[ROWS], inc[ROWS];
 #pragma unroll
-                    for (int k = 0; k < ROWS; ++k)
-                        incl[k] = (lane + 32 * k < n) ? eq5_weight(dv[k] - dmin, beta) : 0ull;
+                    for (int k = 0; k < ROWS; ++k) {
+                        const float w = ex2_approx(__int2float_rn(dv[k]) * kb);
+                        wk[k] = lane + 32 * k < n ? w : 0.0f;
+                        inc[k] = wk[k];
+                    }
 #pragma unroll
                     for (int o = 1; o < 32; o <<= 1) {
 #pragma unroll
                         for (int k = 0; k < ROWS; ++k) {
-                            const unsigned long long y = __shfl_up_sync(kFull, incl[k], o);
-                            if (lane >= o) incl[k] += y;
+                            const float y = __shfl_up_sync(kFull, inc[k], o);
+                            if (lane >= o) inc[k] += y;
                         }
                     }
-                    unsigned long long total = 0;
+                    float ftot = 0.0f;
 #pragma unroll
                     for (int k = 0; k < ROWS; ++k) {
-                        tot[k] = __shfl_sync(kFull, incl[k], 31);
-                        total += tot[k];
+                        const float tk = __shfl_sync(kFull, inc[k], 31);
+                        inc[k] += ftot;
+                        ftot += tk;
                     }
-                    const unsigned long long tdraw = __umul64hi(draw, total);
-                    int js = i, dsel = 0;
-                    unsigned long long off = 0;
-                    bool found = false;
+                    const float tt = __uint2float_rn(draw_hi >> 8) * 5.9604644775390625e-08f * ftot;
+                    const float mg = ftot < kDrawLimit ? kDrawMargin * ftot : __int_as_float(0x7FC00000);
+                    int kk = -1, dsel = 0;
 #pragma unroll
-                    for (int k = 0; k < ROWS; ++k) {
-                        if (!found && tdraw < off + tot[k]) {  // uniform across the warp
-                            const unsigned ball = __ballot_sync(kFull, off + incl[k] > tdraw);
-                            const int src = __ffs(ball) - 1;
-                            js = 32 * k + src;
-                            dsel = __shfl_sync(kFull, dv[k], src);
-                            found = true;
+                    for (int k = 0; k < ROWS; ++k)
+                        if (tt - mg >= inc[k] - wk[k] && tt + mg < inc[k]) {
+                            kk = k;
+                            dsel = dv[k];
                         }
-                        off += tot[k];
+                    int js = i;
+                    const unsigned ball = __ballot_sync(kFull, kk >= 0);
+                    if (ball) {
+                        const int src = __ffs(ball) - 1;
+                        js = 32 * __shfl_sync(kFull, kk, src) + src;
+                        dsel = __shfl_sync(kFull, dsel, src);
+                    } else {
+                        const unsigned long long draw = ((unsigned long long)draw_hi << 32) |
+                                                        (unsigned long long)__shfl_sync(kFull, rw.x, q);
+                        int lmin = 0x7FFFFFFF;
+#pragma unroll
+                        for (int k = 0; k < ROWS; ++k)
+                            if (lane + 32 * k < n) lmin = min(lmin, dv[k]);
+                        const int dmin = __reduce_min_sync(kFull, lmin);
+                        unsigned long long incl[ROWS], tot[ROWS];
+#pragma unroll
+                        for (int k = 0; k < ROWS; ++k)
+                            incl[k] = (lane + 32 * k < n) ? eq5_weight(dv[k] - dmin, beta) : 0ull;
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+#pragma unroll
+                            for (int k = 0; k < ROWS; ++k) {
+                                const unsigned long long y = __shfl_up_sync(kFull, incl[k], o);
+                                if (lane >= o) incl[k] += y;
+                            }
+                        }
+                        unsigned long long total = 0;
+#pragma unroll
+                        for (int k = 0; k < ROWS; ++k) {
+                            tot[k] = __shfl_sync(kFull, incl[k], 31);
+                            total += tot[k];
+                        }
+                        const unsigned long long tdraw = __umul64hi(draw, total);
+                        unsigned long long off = 0;
+                        bool found = false;
+                        dsel = 0;
+#pragma unroll
+                        for (int k = 0; k < ROWS; ++k) {
+                            if (!found && tdraw < off + tot[k]) {  // uniform across the warp
+                                const unsigned hit = __ballot_sync(kFull, off + incl[k] > tdraw);
+                                const int src = __ffs(hit) - 1;
+                                js = 32 * k + src;
+                                dsel = __shfl_sync(kFull, dv[k], src);
+                                found = true;
+                            }
+                            off += tot[k];
+                        }
                     }
                     if (lane == 0) {
                         pj[i] = js;
@@ -1120,9 +1290,7 @@ __device__ __forceinline__ void run_replica(const SweepArgs &a, int part_arg, in
             const int cnt = min(32, n - i0);
             for (int ii = 0; ii < cnt; ++ii) {
                 const int i = i0 + ii;
-                const unsigned long long draw =
-                    ((unsigned long long)__shfl_sync(kFull, rw.y, ii) << 32) |
-                    (unsigned long long)__shfl_sync(kFull, rw.x, ii);
+                const uint32_t draw_hi = __shfl_sync(kFull, rw.y, ii);
                 const int fa = sp[i];
                 const int hi = sh[i];
                 const DT *Di = sD + i * dn;
@@ -1140,7 +1308,6 @@ __device__ __forceinline__ void run_replica(const SweepArgs &a, int part_arg, in
                 }
 
                 // ---- gather: Eq. 3 for every candidate j
-                int lmin = 0x7FFFFFFF;
                 int dself = 0;  // MAXK = 1: this thread's energy, handed to the draw in a register
 #pragma unroll
                 for (int k = 0; k < MAXK; ++k) {
@@ -1193,12 +1360,13 @@ __device__ __forceinline__ void run_replica(const SweepArgs &a, int part_arg, in
                             sv[j] = d;
                         else
                             dself = d;
-                        lmin = min(lmin, d);
                     }
                 }
                 const int nxt = i + 1 < n ? i + 1 : 0;  // the next update's location
                 if constexpr (TG) prefetch(nxt);
-                const int3 sel = eq5_draw<MAXK, WPR>(sv, sp, n, t, lmin, dself, myp, beta, draw, bar, gs);
+                const int3 sel = eq5_draw<MAXK, WPR>(
+                    sv, sp, n, t, dself, myp, beta, draw_hi, [&]() { return __shfl_sync(kFull, rw.x, ii); },
+                    draw_tag(i, s), bar, gs);
                 const int js = sel.x, dstar = sel.y;
                 if (js == i) continue;
 
