@@ -147,9 +147,10 @@ int pdit_set_replicas_per_cta(pdit_qap *h, int g);
 
 /*
  * pdit_launch_shape -- the sweep-kernel launch a call with `replicas` chains
- * would use: shape[0] warps per replica, [1] candidates per thread, [2]
+ * would use: shape[0] warps per replica (1 also where 16 threads run one,
+ * two replicas to a warp), [1] candidates per thread, [2]
  * replicas per CTA, [3] CTAs, [4] 1 if the influence tables live in shared
- * memory (0: global memory; 2: no table, the dot-product kernel of
+ * memory (0: global memory; 2: no table, the product kernels of
  * pdit_set_influence), [5] dynamic shared memory bytes per CTA.
  * [6] pending rank-1 terms held before the influence table is rewritten (1 =
  * after each swap; 4 or 16).
@@ -180,7 +181,10 @@ int pdit_launch_shape(const pdit_qap *h, int replicas, int *shape);
  *                             instances whose D and F entries all lie in
  *                             -128..127, in the sequential modes, without
  *                             the table dump (PDIT_ENOTSUP otherwise, at the
- *                             next call). Two-level-flow instances keep the
+ *                             next call). Above 32 locations, zero diagonals
+ *                             and entries in 0..127 form the products of many
+ *                             replicas on the tensor cores, from D and F
+ *                             themselves and no matrix per replica. Two-level-flow instances keep the
  *                             flow-class kernel unless pdit_set_class_update
  *                             turns it off.
  *   PDIT_INFLUENCE_AUTO     : products where eligible and where shared

@@ -28,6 +28,7 @@ struct pdit_qap {
     int cls_f = 0;
     long long cls_e0 = 0;
     uint8_t *dx = nullptr;  // x_c on the device
+    int nonneg = 0;         // every entry of D and F >= 0
     int packed_ok = 0;      // max-min of D and of F <= 127: swap factors fit int8
     std::vector<int32_t> hD, hF;
     std::vector<uint8_t> cls_x;  // class bit of every facility (two-level flows)
@@ -94,6 +95,7 @@ int stage_stride(int n, int dt) {
 struct Plan {
     int maxk = 1, wpr = 1, pk = 1;
     bool tsmem = true, cls = false, dot = false;
+    bool mm = false;  // with dot: the tensor-core product kernel (pdit_mma.cu)
     int stride = 0, sv_len = 0, cupim_off = 0, v2_off = 0, rc_off = 0, dstride = 0;
     size_t table_elems = 0;  // int32 entries of one replica's saved table (workspace)
     size_t df_bytes = 0, group_bytes = 0, smem = 0;
@@ -362,6 +364,35 @@ int make_dot_plan(const pdit_qap *h, int replicas, int wpr, Plan *p, size_t rese
     return PDIT_OK;
 }
 
+// Whether an instance can run the tensor-core product kernel: symmetric, zero
+// diagonals, every entry of D and F in 0..127.
+bool mm_eligible(const pdit_qap *h) { return !h->asym && h->zero_diag && h->dt_bytes == 1 && h->nonneg; }
+
+// Launch shape of the tensor-core product kernel: its thread mapping and
+// shared memory are fixed by n (MmInfo); replicas per CTA spread the call
+// over the GPU.
+int make_mm_plan(const pdit_qap *h, int replicas, Plan *p, size_t reserve = 0) {
+    pdit::MmInfo info{};
+    const int e = pdit::mm_query(h->n, &info);
+    if (e != 0) return cuda_fail((cudaError_t)e, "occupancy query");
+    if (info.blocks_per_sm < 1 || info.smem + reserve > h->smem_optin) return PDIT_ENOTSUP;
+    p->dot = p->mm = true;
+    p->tsmem = true;
+    p->pk = 1;
+    p->wpr = 1;
+    p->maxk = info.k;
+    p->table_elems = 0;
+    p->threads = info.threads;
+    p->smem = info.smem;
+    const int most = h->force_groups > 0 ? std::min(info.slots, h->force_groups) : info.slots;
+    // One CTA per SM while a call needs no more than half of a CTA's slots.
+    int ctas = h->num_sms;
+    if ((replicas + ctas - 1) / ctas > most / 2) ctas *= info.blocks_per_sm;
+    p->groups = std::max(1, std::min(most, (replicas + ctas - 1) / ctas));
+    p->grid = std::min(ctas, (replicas + p->groups - 1) / p->groups);
+    return PDIT_OK;
+}
+
 // Whether an instance can run the dot-product kernel: symmetric, every entry
 // of D and F in a signed byte (dp4a operands).
 bool dot_eligible(const pdit_qap *h) { return !h->asym && h->dt_bytes == 1; }
@@ -386,6 +417,19 @@ int auto_dot_plan(const pdit_qap *h, int replicas, Plan *p, size_t reserve) {
     return make_dot_plan(h, replicas, h->force_wpr, p, reserve);
 }
 
+// The product kernel of a call: tensor-core products where the instance
+// allows them and no wider mapping than a warp per replica is asked for, else
+// the dot-product kernel. `any`: also where the automatic rule prefers the
+// table kernels.
+int product_plan(const pdit_qap *h, int replicas, Plan *p, size_t reserve, bool any) {
+    if (mm_eligible(h) && h->force_wpr <= 1 && h->n > 32) {
+        const int rc = make_mm_plan(h, replicas, p, reserve);
+        if (rc != PDIT_ENOTSUP) return rc;
+        *p = Plan();
+    }
+    return any ? make_dot_plan(h, replicas, h->force_wpr, p, reserve) : auto_dot_plan(h, replicas, p, reserve);
+}
+
 // Whether a call runs the dot-product kernel: an eligible instance in a
 // sequential mode, without a request for the table dump or for table-kernel
 // knobs (pending terms, table placement), unless the handle asks for it.
@@ -400,10 +444,10 @@ int plan_for(const pdit_qap *h, const pdit_opts *o, Plan *p) {
     if (use_class_path(h, o)) return make_class_plan(h, o->replicas, h->force_wpr, p);
     if (h->force_infl == PDIT_INFLUENCE_PRODUCTS) {
         if (!dot_eligible(h) || o->mode == PDIT_MODE_CUPIM || o->tables) return PDIT_ENOTSUP;
-        return make_dot_plan(h, o->replicas, h->force_wpr, p);
+        return product_plan(h, o->replicas, p, 0, true);
     }
     if (use_dot_path(h, o)) {
-        const int rc = auto_dot_plan(h, o->replicas, p, 0);
+        const int rc = product_plan(h, o->replicas, p, 0, false);
         if (rc != PDIT_ENOTSUP) return rc;
         *p = Plan();  // no suitable dot shape: the table kernels
     }
@@ -475,6 +519,7 @@ int parts_of(const pdit_opts *o, const Plan &p, int span) {
 // kept between calls by the server, the dot kernel's permuted flow matrix;
 // either kernel's table between the parts of a launch).
 bool needs_tables(const pdit_opts *o, const Plan &p, bool persist = false, bool whole = false) {
+    if (p.mm) return false;  // its state is the permutation and the energies
     return persist || o->mode == PDIT_MODE_PT || (!p.dot && !p.tsmem) || (!whole && may_split(o, p));
 }
 
@@ -766,6 +811,7 @@ int qap_prepare(int n, const int32_t *D, const int32_t *F, pdit_qap **out) {
         h->cls_f = (int)fcls;
         h->cls_e0 = f0 * dsum;  // D's diagonal is zero
     }
+    h->nonneg = dlo >= 0 && flo >= 0 ? 1 : 0;
     h->packed_ok = (dhi - dlo <= 127 && fhi - flo <= 127) ? 1 : 0;
     const int64_t mx = std::max(maxd, maxf);
     h->dt_bytes = mx <= 127 ? 1 : (mx <= 32767 ? 2 : 4);
@@ -993,6 +1039,7 @@ int pdit_anneal_ex(pdit_qap *h, const pdit_opts *o) {
             PDIT_CK(cudaMemsetAsync(w.queue, 0, sizeof(int32_t), st));
             if (a.segments > 1) PDIT_CK(cudaMemsetAsync(w.seg_done, 0, sizeof(int32_t) * R, st));
             const int e = plan.cls ? class_launch(h->dt_bytes, plan, a, st)
+                        : plan.mm  ? pdit::mm_launch(a, plan.grid, st)
                         : plan.dot ? pdit::dot_launch(plan.maxk, plan.wpr, a, plan.grid, plan.threads, plan.smem, st)
                                    : sweep_launch(h->dt_bytes, h->asym != 0, plan, a, st);
             if (e != 0) return cuda_fail((cudaError_t)e, "sweep kernel launch");
@@ -1122,7 +1169,7 @@ int pdit_autotune(pdit_qap *h, int replicas, const float *beta, int sweeps, int 
     auto plan_ok = [&](const Knobs &k, Plan *p) {
         set(k);
         if (cls) return make_class_plan(h, replicas, k.wpr, p) == PDIT_OK;
-        if (k.infl == PDIT_INFLUENCE_PRODUCTS) return make_dot_plan(h, replicas, k.wpr, p) == PDIT_OK;
+        if (k.infl == PDIT_INFLUENCE_PRODUCTS) return product_plan(h, replicas, p, 0, true) == PDIT_OK;
         return make_plan(h, replicas, k.wpr, k.pk, p) == PDIT_OK;
     };
     // Candidates: the table placement (a caller's choice, else the built-in

@@ -157,9 +157,10 @@ __device__ __forceinline__ uint4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_
 // proceed in parallel: an x beyond 40 (or not a number) is replaced by 0 for
 // the arithmetic and its weight is zeroed at the end; every other x takes
 // exactly the operations above.
+// eq5_weight_f takes dE - dE_min as the binary32 nearest to the integer.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ unsigned long long eq5_weight(int shifted_de, float beta) {
-    const float x0 = __fmul_rn(__int2float_rn(shifted_de), beta);
+__device__ __forceinline__ unsigned long long eq5_weight_f(float shifted_de, float beta) {
+    const float x0 = __fmul_rn(shifted_de, beta);
     const bool live = x0 <= 40.0f;
     const float x = live ? x0 : 0.0f;
     const float t = __fadd_rn(__fmul_rn(x, 1.44269502f), 0.5f);
@@ -185,6 +186,10 @@ __device__ __forceinline__ unsigned long long eq5_weight(int shifted_de, float b
     const unsigned long long m30 = (unsigned long long)((bits & 0x7FFFFFu) | 0x800000u) << 30;
     const int s = live ? 127 - (int)(bits >> 23) + k : 63;
     return m30 >> s;
+}
+
+__device__ __forceinline__ unsigned long long eq5_weight(int shifted_de, float beta) {
+    return eq5_weight_f(__int2float_rn(shifted_de), beta);
 }
 
 __device__ __forceinline__ int warp_min(int v) {
@@ -1727,5 +1732,15 @@ int dot_launch(int maxk, int wpr, const SweepArgs &a, int grid, int threads, siz
 int dot_batch_blocks_per_sm(int maxk, int wpr, int threads, size_t smem, int *blocks);
 int dot_batch_launch(int maxk, int wpr, const SweepArgs *descs, const BatchUnit *units, int nunits, int *queue,
                      int grid, int threads, size_t smem, cudaStream_t stream);
+
+// Tensor-core product kernel (pdit_mma.cu): symmetric instances with zero
+// diagonals and entries in 0..127; one compiled kernel per range of n.
+// Return a cudaError_t value.
+struct MmInfo {
+    int threads, slots, lanes, k, blocks_per_sm;  // slots: replicas per CTA; lanes: threads per replica
+    size_t smem;
+};
+int mm_query(int n, MmInfo *info);
+int mm_launch(const SweepArgs &a, int grid, cudaStream_t stream);
 
 }  // namespace pdit
