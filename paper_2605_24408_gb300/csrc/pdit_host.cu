@@ -96,6 +96,7 @@ struct Plan {
     int maxk = 1, wpr = 1, pk = 1;
     bool tsmem = true, cls = false, dot = false;
     bool mm = false;  // with dot: the tensor-core product kernel (pdit_mma.cu)
+    int lanes = 32;   // its threads per replica
     int stride = 0, sv_len = 0, cupim_off = 0, v2_off = 0, rc_off = 0, dstride = 0;
     size_t table_elems = 0;  // int32 entries of one replica's saved table (workspace)
     size_t df_bytes = 0, group_bytes = 0, smem = 0;
@@ -381,6 +382,7 @@ int make_mm_plan(const pdit_qap *h, int replicas, Plan *p, size_t reserve = 0) {
     p->pk = 1;
     p->wpr = 1;
     p->maxk = info.k;
+    p->lanes = info.lanes;
     p->table_elems = 0;
     p->threads = info.threads;
     p->smem = info.smem;
@@ -462,12 +464,12 @@ int batch_plan(const pdit_qap *h, Plan *p, size_t reserve) {
     if (!h->cls || !h->use_cls) {
         if (h->force_infl == PDIT_INFLUENCE_PRODUCTS) {
             if (!dot_eligible(h)) return PDIT_ENOTSUP;
-            return make_dot_plan(h, 1 << 28, h->force_wpr, p, reserve);
+            return product_plan(h, 1 << 28, p, reserve, true);
         }
         pdit_opts o;
         pdit_opts_init(&o);
         if (use_dot_path(h, &o)) {
-            const int rc = auto_dot_plan(h, 1 << 28, p, reserve);
+            const int rc = product_plan(h, 1 << 28, p, reserve, false);
             if (rc != PDIT_ENOTSUP) return rc;
             *p = Plan();
         }
@@ -1033,6 +1035,7 @@ int pdit_anneal_ex(pdit_qap *h, const pdit_opts *o) {
         // kernel or mode ran before it.
         a.table_in = (pt && !first) ? 1 : 0;
         a.table_out = (pt && next < se) ? 1 : 0;
+        a.audit = next == se ? 1 : 0;
         a.dump = (next == se) ? o->tables : nullptr;
         a.segments = parts_of(o, plan, next - s);
         if (!(first && resume && s == se)) {
@@ -1485,7 +1488,8 @@ struct BatchOut {
 
 struct BatchClass {
     int dt = 1, maxk = 1, wpr = 1, pk = 1;
-    bool tsmem = true, asym = false, dot = false;
+    bool tsmem = true, asym = false, dot = false, mm = false;
+    int lanes = 32, n = 0;  // mm: threads per replica, the size of one of its instances
     int threads = 32, grid = 1, nunits = 0;
     size_t smem = 0;
     std::vector<int> items;
@@ -1502,6 +1506,7 @@ int batch_blocks_t(const BatchClass &c, int *blocks) {
 }
 
 int batch_blocks(const BatchClass &c, int *blocks) {
+    if (c.mm) return pdit::mm_batch_blocks_per_sm(c.n, blocks);
     if (c.dot) return pdit::dot_batch_blocks_per_sm(c.maxk, c.wpr, c.threads, c.smem, blocks);
     return c.asym ? batch_blocks_t<true>(c, blocks) : batch_blocks_t<false>(c, blocks);
 }
@@ -1519,6 +1524,7 @@ int batch_launch_t(const BatchClass &c, const pdit::SweepArgs *descs, int *queue
 }
 
 int batch_launch(const BatchClass &c, const pdit::SweepArgs *descs, int *queue) {
+    if (c.mm) return pdit::mm_batch_launch(c.n, descs, c.d_units, c.nunits, queue, c.grid, c.stream);
     if (c.dot)
         return pdit::dot_batch_launch(c.maxk, c.wpr, descs, c.d_units, c.nunits, queue, c.grid, c.threads, c.smem,
                                       c.stream);
@@ -1527,13 +1533,17 @@ int batch_launch(const BatchClass &c, const pdit::SweepArgs *descs, int *queue) 
 
 // Same compiled kernel shape.
 bool same_class(const BatchClass &x, int dt, bool asym, const Plan &p) {
+    if (x.mm || p.mm) return x.mm == p.mm && x.maxk == p.maxk && x.lanes == p.lanes;
     if (x.dot || p.dot) return x.dot == p.dot && x.maxk == p.maxk && x.wpr == p.wpr;
     return x.dt == dt && x.asym == asym && x.maxk == p.maxk && x.wpr == p.wpr && x.pk == p.pk && x.tsmem == p.tsmem;
 }
 
 // A new shape class for plan p.
-BatchClass class_for(int dt, bool asym, const Plan &p) {
+BatchClass class_for(int dt, bool asym, const Plan &p, int n) {
     BatchClass x;
+    x.mm = p.mm;
+    x.lanes = p.lanes;
+    x.n = n;
     x.dt = dt;
     x.asym = asym;
     x.dot = p.dot;
@@ -1542,6 +1552,35 @@ BatchClass class_for(int dt, bool asym, const Plan &p) {
     x.pk = p.pk;
     x.tsmem = p.tsmem;
     return x;
+}
+
+// Replicas per work unit of the tensor-core product kernel in a
+// multi-instance launch. A unit of 16 is the most efficient (one of 8 takes
+// about 0.78 of its time, one of 4 about 0.66), but a launch lasts at least as
+// long as its longest unit: where a unit of 16 would outlast the whole
+// launch spread evenly over the GPU, its instance takes smaller ones.
+struct UnitLoad {
+    const Plan *plan;
+    int n, replicas;
+    double sweeps;
+};
+double unit_cost(const UnitLoad &u) {
+    // clocks per update step of a full block, measured: about 3600 at N =
+    // 100 (two CTAs per SM), 6000 at N = 256 (one)
+    return u.sweeps * u.n * (1000.0 + (u.plan->lanes == 16 ? 26.0 : 20.0) * u.n);
+}
+std::vector<int> unit_groups(const std::vector<UnitLoad> &loads, int num_sms) {
+    double total = 0.0;
+    for (const UnitLoad &u : loads)
+        if (u.plan->mm) total += unit_cost(u) * u.replicas / 16.0 * (u.plan->lanes == 16 ? 0.5 : 1.0) / num_sms;
+    std::vector<int> g;
+    for (const UnitLoad &u : loads) {
+        int k = u.plan->groups;
+        if (u.plan->mm)
+            while (k > 4 && unit_cost(u) * (0.55 + 0.45 * k / 16.0) > total) k = (k + 1) / 2;
+        g.push_back(k);
+    }
+    return g;
 }
 
 // Per instance: reset its time-to-target outputs and stop flag.
@@ -1691,8 +1730,16 @@ int pdit_batch_create(const pdit_batch_item *items, int count, uint32_t flags, p
         ws_off[k] = ws_total;
         ws_total += align_up(carve(h, &o, plans[k], nullptr, false, true).bytes, kAlign);  // batches: whole calls
     }
-    // Shape classes.
-    for (int k = 0; k < count; ++k) {
+    std::vector<UnitLoad> loads;
+    for (int k = 0; k < count; ++k)
+        loads.push_back({&plans[k], items[k].qap->n, items[k].replicas, (double)items[k].sweeps});
+    const std::vector<int> groups = unit_groups(loads, items[0].qap->num_sms);
+    for (int k = 0; k < count; ++k) plans[k].groups = groups[k];
+    // Shape classes, the larger sizes first: the longest units start first.
+    std::vector<int> by_size((size_t)count);
+    for (int k = 0; k < count; ++k) by_size[k] = k;
+    std::stable_sort(by_size.begin(), by_size.end(), [&](int u, int v) { return items[u].qap->n > items[v].qap->n; });
+    for (int k : by_size) {
         const Plan &p = plans[k];
         const int dt = items[k].qap->dt_bytes;
         const bool asym = items[k].qap->asym != 0;
@@ -1700,7 +1747,7 @@ int pdit_batch_create(const pdit_batch_item *items, int count, uint32_t flags, p
         for (size_t c = 0; c < b->classes.size(); ++c)
             if (same_class(b->classes[c], dt, asym, p)) found = (int)c;
         if (found < 0) {
-            b->classes.push_back(class_for(dt, asym, p));
+            b->classes.push_back(class_for(dt, asym, p, items[k].qap->n));
             found = (int)b->classes.size() - 1;
         }
         BatchClass &x = b->classes[found];
@@ -1743,6 +1790,7 @@ int pdit_batch_create(const pdit_batch_item *items, int count, uint32_t flags, p
         a.mode = 0;
         a.beta = it.beta;
         a.fresh = 1;
+        a.audit = 1;
         a.perm = w.perm;
         a.best_perm = w.best_perm;
         a.energy = w.energy;
@@ -2210,23 +2258,32 @@ int pdit_server_tick(pdit_server *s, int *active, int *queued) {
         int rc = poll(s, b, true);  // the buffer's previous copies are done
         if (rc) return rc;
         size_t nunits = 0, nres = 0;
-        for (ServerRequest *r : s->active) {
-            nunits += (size_t)(r->replicas + r->plan.groups - 1) / r->plan.groups;
+        std::vector<UnitLoad> loads;
+        std::vector<int> by_size;  // larger sizes first: the longest units start first
+        for (int k = 0; k < na; ++k) {
+            const ServerRequest *r = s->active[k];
+            loads.push_back({&r->plan, r->n, r->replicas, (double)std::min(s->slice, r->sweeps - r->done_sweeps)});
+            by_size.push_back(k);
             nres += r->done_sweeps + s->slice >= r->sweeps ? 1 : 0;
         }
+        std::stable_sort(by_size.begin(), by_size.end(),
+                         [&](int x, int y) { return s->active[x]->n > s->active[y]->n; });
+        const std::vector<int> groups = unit_groups(loads, s->active[0]->qap->num_sms);
+        for (int k = 0; k < na; ++k) nunits += (size_t)(s->active[k]->replicas + groups[k] - 1) / groups[k];
         rc = grow(s, b, (size_t)na, nunits, nres);
         if (rc) return rc;
         std::vector<BatchClass> cls;
         std::vector<std::vector<int>> members;
         std::vector<ServerRequest *> finishing;
         int nout = 0;
-        for (int k = 0; k < na; ++k) {
+        for (int k : by_size) {
             ServerRequest *r = s->active[k];
             const Plan &p = r->plan;
             const int end = std::min(r->sweeps, r->done_sweeps + s->slice);
             pdit::SweepArgs &a = b.h_descs[k];
             a = pdit::SweepArgs{};
             fill_shape(a, r->qap, p);
+            a.groups = groups[k];
             a.replicas = r->replicas;
             a.sweep_begin = r->done_sweeps;
             a.sweep_end = end;
@@ -2237,6 +2294,7 @@ int pdit_server_tick(pdit_server *s, int *active, int *queued) {
             a.fresh = r->done_sweeps == 0 ? 1 : 0;
             a.table_in = a.fresh ? 0 : 1;       // resume from the saved state
             a.table_out = end < r->sweeps ? 1 : 0;  // save it for the next slice
+            a.audit = end >= r->sweeps ? 1 : 0;
             a.perm = r->w.perm;
             a.best_perm = r->w.best_perm;
             a.energy = r->w.energy;
@@ -2256,7 +2314,7 @@ int pdit_server_tick(pdit_server *s, int *active, int *queued) {
             for (size_t c = 0; c < cls.size(); ++c)
                 if (same_class(cls[c], dt, asym, p)) found = (int)c;
             if (found < 0) {
-                cls.push_back(class_for(dt, asym, p));
+                cls.push_back(class_for(dt, asym, p, r->n));
                 members.emplace_back();
                 found = (int)cls.size() - 1;
             }
@@ -2281,7 +2339,7 @@ int pdit_server_tick(pdit_server *s, int *active, int *queued) {
             cls[c].d_units = s->d_units + u;
             const size_t u0 = u;
             for (int k : order)
-                for (int r0 = 0; r0 < s->active[k]->replicas; r0 += s->active[k]->plan.groups)
+                for (int r0 = 0; r0 < s->active[k]->replicas; r0 += groups[k])
                     b.h_units[u++] = pdit::BatchUnit{k, r0};
             cls[c].nunits = (int)(u - u0);
             cls[c].stream = s->classes[c].stream;

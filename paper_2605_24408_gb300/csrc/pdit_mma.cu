@@ -26,11 +26,6 @@
 // t*K + k. Steps of one update: the gathers (each replica's threads), a CTA
 // barrier, the products (each warp holds its rows of D or F for all
 // replicas), a barrier, and energies, draw and swap (each replica's threads).
-//
-// Bound: shared-memory wavefronts (93 per update at N = 100, 69% of the
-// pipe's cycles), then the latency of the three phases. Measured at N = 100,
-// 4096 replicas: 2.13e9 updates/s against 1.22e9 with the dot-product kernel;
-// N = 256, 2048 replicas: 7.4e8 against 1.8e8 with the table kernels.
 #include "pdit_sweep.cuh"
 
 namespace pdit {
@@ -45,19 +40,26 @@ struct MmShape {
     static constexpr int R = 16;                  // replica slots per CTA
     static constexpr int JT = (MT + NW / 2 - 1) / (NW / 2);  // row tiles per warp
     static constexpr bool REGS = MT <= 8;         // the warp's rows stay in registers
-    // Row strides. Tables, bytes: 16 x odd, so that 8 rows x 16 bytes read by
-    // a warp fall in 32 distinct banks. Vectors, bytes: 32 mod 64, the same
-    // for 64-bit reads. Results, floats: 4 mod 16, so that the four column
-    // pairs of a fragment store and the replicas of one warp (r, r + 4) hit
-    // distinct banks.
-    static constexpr int DS = 16 * (MT | 1);
+    // Row strides. Tables, bytes: 256 where the fragments are read once, so
+    // that a gather's address is its row's with the byte index for the low
+    // byte (one byte permute); else 16 x odd, so that 8 rows x 16 bytes read
+    // by a warp fall in 32 distinct banks. Vectors, bytes: 32 mod 64, the same
+    // for 64-bit reads, and the two replicas of a warp, 2 rows apart, store to
+    // disjoint banks. Results, floats: 4 mod 16, so that the four column pairs
+    // of a fragment store hit distinct banks and the two replicas of a warp,
+    // 4 rows apart (crow), read disjoint ones.
+    static constexpr int DS = REGS ? 256 : 16 * (MT | 1);
     static constexpr int VS = 32 * (MT | 1);
     static constexpr int CS = NP + 4;
     static constexpr int PS = 8 * LPR;            // permutation bytes of a replica (8 per thread)
-    // shared memory
+    // shared memory (the tables first: their rows are 256-byte aligned)
     static constexpr int oD = 0, oF = oD + NP * DS, oVq = oF + NP * DS, oVg = oVq + R * VS, oC = oVg + R * VS,
                          oR = oC + 4 * R * CS, oH = oR + 4 * R * CS, oP = oH + 4 * R * CS, oI = oP + R * PS,
                          oDr = oI + R * PS, oX = oDr + 8 * NP, bytes = oX + 16;
+    // result row of the replica in vector row v: bits 1 and 2 of v trade places
+    __host__ __device__ static constexpr int crow(int v) {
+        return LPR == 32 ? v : (v & ~6) | ((v & 2) << 1) | ((v & 4) >> 1);
+    }
     // Orders. Locations (rows and columns of D, the vector q, the results C,
     // h): t*K + k at pos(t, k), pairs of a thread's locations together, so
     // that it moves two as one word. Facilities (F, the vector g, the
@@ -102,6 +104,29 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
     return d;
 }
 __device__ __forceinline__ float2 two(float v) { return make_float2(v, v); }
+
+// Loads at 32-bit shared-window addresses (volatile: they stay on their side
+// of the barriers).
+__device__ __forceinline__ int lds_u8(uint32_t a) {
+    int v;
+    asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ float lds_f32(uint32_t a) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ float2 lds_f64(uint32_t a) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ uint2 lds_u64(uint32_t a) {
+    uint2 v;
+    asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+    return v;
+}
 
 // Byte k of the eight in v.
 __device__ __forceinline__ int byte8(const uint2 v, int k) {
@@ -157,6 +182,15 @@ __device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], c
 // The 16 x 16 fragment of rows row0.. of a table at depth step s. Depth order
 // within a step: a thread's four consecutive bytes are the fragment's (2q,
 // 2q + 1) and (2q + 8, 2q + 9), as in the vectors.
+// Address of entry byte8(v, k) of the table row at `row`.
+template <class S>
+__device__ __forceinline__ uint32_t entry(uint32_t row, const uint2 v, int k) {
+    if constexpr (S::DS == 256)
+        return __byte_perm(k < 4 ? v.x : v.y, row, 0x7650 | (k & 3));
+    else
+        return row + (uint32_t)byte8(v, k);
+}
+
 template <int DS>
 __device__ __forceinline__ void mm_frag(const uint8_t *tab, int row0, int s, int lane, uint32_t (&a)[4]) {
     const uint8_t *p = tab + (row0 + (lane >> 2)) * DS + 16 * s + 4 * (lane & 3);
@@ -184,7 +218,7 @@ __device__ __forceinline__ void mm_stage(const int32_t *D, const int32_t *F, int
     }
     __syncthreads();
     if constexpr (S::REGS) {
-        const int w = threadIdx.x >> 5;
+        const int w = __shfl_sync(kFull, threadIdx.x >> 5, 0);
         const uint8_t *tab = sm + (w < S::NW / 2 ? S::oD : S::oF);
 #pragma unroll
         for (int jt = 0; jt < S::JT; ++jt) {
@@ -197,8 +231,8 @@ __device__ __forceinline__ void mm_stage(const int32_t *D, const int32_t *F, int
 
 // This warp's row tiles of D x [q] or F x [g] for NT x 8 replicas.
 template <class S, int NT>
-__device__ __forceinline__ void mm_products(unsigned char *sm, const uint32_t (&A)[S::JT][S::REGS ? S::MT : 1][4]) {
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+__device__ __forceinline__ void mm_products(unsigned char *sm, int w, const uint32_t (&A)[S::JT][S::REGS ? S::MT : 1][4]) {
+    const int lane = threadIdx.x & 31;
     const int g = lane >> 2, q = lane & 3;
     const bool second = w >= S::NW / 2;
     const int m0 = w % (S::NW / 2);
@@ -232,14 +266,15 @@ __device__ __forceinline__ void mm_products(unsigned char *sm, const uint32_t (&
             }
         }
     }
-    float *out = reinterpret_cast<float *>(sm + (second ? S::oR : S::oC));
+    // columns 2q and 2q + 1 of a tile go to result rows crow(2q) and, one on, crow(2q + 1)
+    float *out = reinterpret_cast<float *>(sm + (second ? S::oR : S::oC)) + S::crow(2 * q) * S::CS + g;
 #pragma unroll
     for (int jt = 0; jt < S::JT; ++jt) {
         const int m = m0 + jt * (S::NW / 2);
         if (m >= S::MT) break;
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
-            float *o = out + (8 * nt + 2 * q) * S::CS + 16 * m + g;
+            float *o = out + 8 * nt * S::CS + 16 * m;
             o[0] = acc[jt][nt][0];
             o[S::CS] = acc[jt][nt][1];
             o[8] = acc[jt][nt][2];
@@ -248,22 +283,23 @@ __device__ __forceinline__ void mm_products(unsigned char *sm, const uint32_t (&
     }
 }
 
-// p-diagonal entries of this thread's locations, h[x] = sum_y D[x][y]
-// F[p(x)][p(y)], from the replica's permutation bytes (integers).
+// p-diagonal entries of this thread's locations, h[x] = sum_y D[y][x]
+// F[p(y)][p(x)] (symmetric), from the replica's permutation bytes (integers);
+// one row of each table at a time.
 template <class S>
 __device__ __forceinline__ void mm_diagonal(const unsigned char *sm, const uint8_t *pb, int n, int t, int (&h)[S::K]) {
     constexpr int K = S::K;
-    const uint8_t *fr[K];
+    int px[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) {
         h[k] = 0;
-        fr[k] = sm + S::oF + pb[t * 8 + k] * S::DS;
+        px[k] = pb[t * 8 + k];
     }
+#pragma unroll 2
     for (int y = 0; y < n; ++y) {
-        const int py = pb[S::pbyte(y)];
-        const uint8_t *dc = sm + S::oD + S::loc(y);
+        const uint8_t *dr = sm + S::oD + S::loc(y) * S::DS, *fr = sm + S::oF + pb[S::pbyte(y)] * S::DS;
 #pragma unroll
-        for (int k = 0; k < K; ++k) h[k] += (int)dc[S::pos(t, k) * S::DS] * (int)fr[k][py];
+        for (int k = 0; k < K; ++k) h[k] += (int)dr[S::pos(t, k)] * (int)fr[px[k]];
     }
 }
 
@@ -280,32 +316,39 @@ template <class S>
 __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int part, unsigned char *sm,
                                              const uint32_t (&A)[S::JT][S::REGS ? S::MT : 1][4]) {
     constexpr int K = S::K, LPR = S::LPR;
-    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, w = __shfl_sync(kFull, tid >> 5, 0), lane = tid & 31;
     const int half = LPR == 16 ? lane >> 4 : 0;
     const int t = lane & (LPR - 1);
     const unsigned mask = LPR == 32 ? kFull : 0xFFFFu << (16 * half);
     const int n = a.n;
     const int count = min(a.groups, a.replicas - r0);  // replicas of this block
-    // slot of this thread's replica; the two of a warp are 4 apart (row strides)
-    const int slot = LPR == 32 ? w : (w & 3) + 8 * (w >> 2) + 4 * half;
-    const bool live = slot < count;
-    const bool warp_live = LPR == 32 ? live : (w & 3) + 8 * (w >> 2) < count;
-    const int r = r0 + slot;
+    // vector row of this thread's replica; the two of a warp are 2 apart.
+    // More than 8 replicas fill the warps two by two.
+    const int v0 = LPR == 32 ? w : (w & 1) + 4 * (w >> 1);
+    const int slot = v0 + 2 * half;
+    const int idx = LPR == 16 && count > 8 ? 2 * w + half : slot;
+    const bool live = idx < count;
+    const bool warp_live = (LPR == 16 && count > 8 ? 2 * w : v0) < count;
+    const int r = r0 + idx;
     const uint32_t grep = a.rep_base + (uint32_t)r;
-    float *sC = reinterpret_cast<float *>(sm + S::oC) + slot * S::CS;
-    float *sR = reinterpret_cast<float *>(sm + S::oR) + slot * S::CS;
-    float *sH = reinterpret_cast<float *>(sm + S::oH) + slot * S::CS;
+    float *sC = reinterpret_cast<float *>(sm + S::oC) + S::crow(slot) * S::CS;
+    float *sR = reinterpret_cast<float *>(sm + S::oR) + S::crow(slot) * S::CS;
+    float *sH = reinterpret_cast<float *>(sm + S::oH) + S::crow(slot) * S::CS;
     uint8_t *pb = sm + S::oP + slot * S::PS;
     uint8_t *ib = sm + S::oI + slot * S::PS;
     float *drow = reinterpret_cast<float *>(sm + S::oDr);
     volatile int *flag = reinterpret_cast<volatile int *>(sm + S::oX);
+    // shared-window addresses
+    const uint32_t base32 = (uint32_t)__cvta_generic_to_shared(sm);
+    const uint32_t aP = base32 + S::oP + slot * S::PS, aI = aP + (S::oI - S::oP);
+    const uint32_t aC = base32 + S::oC + 4 * S::crow(slot) * S::CS, aR = aC + (S::oR - S::oC), aH = aC + (S::oH - S::oC);
     int32_t *gp = a.perm + (size_t)r * n;
     int32_t *gbp = a.best_perm + (size_t)r * n;
     const bool fresh = part == 0 && a.fresh;
 
     // (|E| <= n^2 127^2 < 2^31)
-    int E = 0, bestE = 0, bsweep = -1;
-    long long acc_moves = 0;
+    // (the best sweep and the accepted swaps stay in global memory)
+    int E = 0, bestE = 0;
     bool reached = false;
     if (warp_live) {
         // ---- permutation: bytes by thread, and its inverse. A slot without
@@ -357,12 +400,14 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
             if (fresh) {
                 E = bestE = esum;
                 for (int m = t; m < n; m += LPR) gbp[m] = tmp[m];
-                if (t == 0) note_target(a, bestE, -1, reached);
+                if (t == 0) {
+                    a.best_sweep[r] = -1;
+                    a.accepted[r] = 0;
+                    note_target(a, bestE, -1, reached);
+                }
             } else {
                 E = (int)__ldcg(a.energy + r);
                 bestE = (int)__ldcg(a.best_energy + r);
-                bsweep = __ldcg(a.best_sweep + r);
-                acc_moves = __ldcg(a.accepted + r);
                 if (E != esum && t == 0) atomicOr(a.status, 1);
             }
         }
@@ -370,9 +415,11 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
     }
     const int s_begin = part_begin(a, part);
     const int s_end = part >= a.segments - 1 ? a.sweep_end : part_begin(a, part + 1);
-    const float beta_fixed = a.sweep_end <= a.sweep_begin || !live ? 0.0f
-                           : a.mode == 1 ? a.beta[a.rung[r]] : a.mode == 2 ? a.beta[r] : 0.0f;
+    auto beta_of = [&](int s) {
+        return a.mode == 1 || a.mode == 2 ? (!live ? 0.0f : a.mode == 1 ? a.beta[a.rung[r]] : a.beta[r]) : a.beta[s];
+    };
     int par = 0;
+    const uint32_t aV = base32 + S::oVq + slot * S::VS + 4 * t;  // this thread's words of q; g at + oVg - oVq
 
     for (int s = s_begin; s < s_end; ++s) {
         if (a.stop) {
@@ -382,86 +429,81 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
             __syncthreads();
             if (*flag) break;
         }
-        const float beta = (a.mode == 1 || a.mode == 2) ? beta_fixed : a.beta[s];
         // (never 0, so that an infinite energy always has weight 0)
-        const float kb = fminf(-beta * kLog2e * kMmScale, -1e-37f);
-        uint32_t rlo = 0, rhi = 0;
+        const float kb = fminf(-beta_of(s) * kLog2e * kMmScale, -1e-37f);
+        uint32_t rhi = 0;  // high words of the draws of LPR locations
         int moves = 0;
         // location i = ti K + ki
         for (int i = 0, ti = 0, ki = 0; i < n; ++i) {
             if ((i & (LPR - 1)) == 0 && warp_live) {
                 // Philox(inst, replica, sweep, location) for the next LPR locations
-                const uint4 rw = philox4x32_10(a.inst, grep, (uint32_t)s, (uint32_t)(i + t), a.key0, a.key1);
-                rlo = rw.x;
-                rhi = rw.y;
+                rhi = philox4x32_10(a.inst, grep, (uint32_t)s, (uint32_t)(i + t), a.key0, a.key1).y;
             }
             const int xi = S::pos(ti, ki);
-            const uint8_t *Drow = sm + S::oD + xi * S::DS;
-            float *dr = drow + par * S::NP;  // 2 D_ij units
+            const uint32_t aDi = base32 + S::oD + xi * S::DS;
+            const uint32_t aDr = base32 + S::oDr + par * 4 * S::NP;  // 2 D_ij units
             uint2 p8 = make_uint2(0, 0);
             int pi = 0, qb[K];
-            const uint8_t *Frow = sm;
+            uint32_t aFi = 0;
             // ---- vectors
-            if (tid < S::NP) dr[tid] = (float)Drow[tid] * (2.0f * kMmUnit);
+            if (tid < S::NP)
+                asm volatile("st.shared.f32 [%0], %1;" ::"r"(aDr + 4 * tid), "f"((float)lds_u8(aDi + tid) * (2.0f * kMmUnit)));
             if (warp_live) {
-                pi = pb[8 * ti + ki];
-                p8 = *reinterpret_cast<const uint2 *>(pb + 8 * t);
-                const uint2 i8 = *reinterpret_cast<const uint2 *>(ib + 8 * t);
-                Frow = sm + S::oF + pi * S::DS;
+                pi = lds_u8(aP + 8 * ti + ki);
+                p8 = lds_u64(aP + 8 * t);
+                const uint2 i8 = lds_u64(aI + 8 * t);
+                aFi = base32 + S::oF + pi * S::DS;
                 int gb[K];
 #pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    gb[k] = Drow[byte8(i8, k)];
-                    qb[k] = Frow[byte8(p8, k)];
-                }
-                unsigned char *vq = sm + S::oVq + slot * S::VS, *vg = sm + S::oVg + slot * S::VS;
+                for (int k = 0; k < K; ++k) gb[k] = lds_u8(entry<S>(aDi, i8, k));
+#pragma unroll
+                for (int k = 0; k < K; ++k) qb[k] = lds_u8(entry<S>(aFi, p8, k));
 #pragma unroll
                 for (int k = 0; k + 1 < K; k += 2) {
-                    *reinterpret_cast<uint32_t *>(vg + k * 2 * LPR + 4 * t) = (uint32_t)gb[k] + 65536u * (uint32_t)gb[k + 1];
-                    *reinterpret_cast<uint32_t *>(vq + k * 2 * LPR + 4 * t) = (uint32_t)qb[k] + 65536u * (uint32_t)qb[k + 1];
+                    const uint32_t g2 = __byte_perm(gb[k], gb[k + 1], 0x5410), q2 = __byte_perm(qb[k], qb[k + 1], 0x5410);
+                    asm volatile("st.shared.b32 [%0], %1;" ::"r"(aV + (S::oVg - S::oVq) + k * 2 * LPR), "r"(g2));
+                    asm volatile("st.shared.b32 [%0], %1;" ::"r"(aV + k * 2 * LPR), "r"(q2));
                 }
                 if constexpr (K & 1) {
-                    *reinterpret_cast<uint16_t *>(vg + (K - 1) * 2 * LPR + 2 * t) = (uint16_t)gb[K - 1];
-                    *reinterpret_cast<uint16_t *>(vq + (K - 1) * 2 * LPR + 2 * t) = (uint16_t)qb[K - 1];
+                    asm volatile("st.shared.b16 [%0], %1;" ::"r"(aV - 2 * t + (S::oVg - S::oVq) + (K - 1) * 2 * LPR),
+                                 "h"((uint16_t)gb[K - 1]));
+                    asm volatile("st.shared.b16 [%0], %1;" ::"r"(aV - 2 * t + (K - 1) * 2 * LPR), "h"((uint16_t)qb[K - 1]));
                 }
             }
             __syncthreads();
             // ---- products
             if (count > 8)
-                mm_products<S, 2>(sm, A);
+                mm_products<S, 2>(sm, w, A);
             else
-                mm_products<S, 1>(sm, A);
+                mm_products<S, 1>(sm, w, A);
             __syncthreads();
             if (warp_live) {
                 // ---- swap energies, half of Eq. 3, up to the common h_i:
                 // I[i][p(j)] + I[j][p(i)] - h_j + 2 D_ij F_ab
-                const float hi = sR[pi];  // I[i][p(i)]
+                const float hi = lds_f32(aR + 4 * pi);  // I[i][p(i)]
                 MmVals<K> e;
-                float hk[K], mq[K], di[K];
+                float hk[K], mq[K];
 #pragma unroll
                 for (int k = 0; k < K; ++k) mq[k] = __int_as_float(0x4B000000 | qb[k]);  // 2^23 + F_ab
 #pragma unroll
                 for (int k = 0; k + 1 < K; k += 2) {
-                    const int x = k * LPR + 2 * t;
-                    const float2 c = *reinterpret_cast<const float2 *>(sC + x);
-                    const float2 h = *reinterpret_cast<const float2 *>(sH + x);
-                    const float2 d = *reinterpret_cast<const float2 *>(dr + x);
-                    const float2 rr = make_float2(sR[byte8(p8, k)], sR[byte8(p8, k + 1)]);
+                    const uint32_t x = 4 * k * LPR + 8 * t;
+                    const float2 c = lds_f64(aC + x);
+                    const float2 h = lds_f64(aH + x);
+                    const float2 d = lds_f64(aDr + x);
+                    const float2 rr = make_float2(lds_f32(aR + 4 * byte8(p8, k)), lds_f32(aR + 4 * byte8(p8, k + 1)));
                     const float2 q = sub2(make_float2(mq[k], mq[k + 1]), two(8388608.0f));
                     const float2 v = fma2(d, q, add2(rr, sub2(c, h)));
                     hk[k] = h.x;
                     hk[k + 1] = h.y;
-                    di[k] = d.x;
-                    di[k + 1] = d.y;
                     e.v[k] = v.x;
                     e.v[k + 1] = v.y;
                 }
                 if constexpr (K & 1) {
                     constexpr int k = K - 1;
-                    const int x = k * LPR + t;
-                    hk[k] = sH[x];
-                    di[k] = dr[x];
-                    e.v[k] = fmaf(di[k], mq[k] - 8388608.0f, sR[byte8(p8, k)] + (sC[x] - hk[k]));
+                    const uint32_t x = 4 * (k * LPR + t);
+                    hk[k] = lds_f32(aH + x);
+                    e.v[k] = fmaf(lds_f32(aDr + x), mq[k] - 8388608.0f, lds_f32(aR + 4 * byte8(p8, k)) + (lds_f32(aC + x) - hk[k]));
                 }
                 // ---- binary32 draw, kept where it is certainly the exact
                 // one (eq5_draw_core): no interval end within m of t
@@ -499,48 +541,45 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
                     kk += (int)((uint32_t)__float_as_int(z) >> 31);
                 }
                 const unsigned ball = __ballot_sync(kFull, base < 0.0f && z > 0.0f && near > mg) & mask;
-                int tj, kj, fb;  // the drawn location tj K + kj and its facility
-                if (ball) {
-                    const int own = __ffs(ball) - 1;
-                    const int v = __shfl_sync(mask, kk | (int)(__byte_perm(p8.x, p8.y, kk) << 8), own);
-                    tj = own & (LPR - 1);
-                    kj = v & 0xFF;
-                    fb = (v >> 8) & 0xFF;
-                } else {
-                    const uint32_t dlo = __shfl_sync(mask, rlo, i & (LPR - 1), LPR);
-                    const int js = mm_exact_draw<K, LPR>(e, n, t, beta, ((unsigned long long)dhi << 32) | dlo, mask);
-                    tj = js / K;
-                    kj = js - tj * K;
-                    fb = pb[8 * tj + kj];
+                // the drawn location tj K + kj and its facility, from its owner
+                int v = __shfl_sync(kFull, (t << 8) | kk | (int)(__byte_perm(p8.x, p8.y, kk) << 16), __ffs(ball) - 1);
+                if (__any_sync(kFull, ball == 0)) {
+                    const uint32_t dlo = philox4x32_10(a.inst, grep, (uint32_t)s, (uint32_t)i, a.key0, a.key1).x;
+                    const int js = mm_exact_draw<K, LPR>(e, n, t, beta_of(s), ((unsigned long long)dhi << 32) | dlo, kFull);
+                    if (ball == 0) {
+                        const int tx = js / K, kx = js - tx * K;
+                        v = (tx << 8) | kx | (lds_u8(aP + 8 * tx + kx) << 16);
+                    }
                 }
-                __syncwarp();
-                // ---- apply the swap i <-> j (facilities fa = p(i), fb = p(j))
+                const int tj = (v >> 8) & 0xFF, kj = v & 0xFF;
+                // ---- apply the swap i <-> j (facilities a = p(i), b = p(j))
                 const bool sw = tj != ti || kj != ki;
                 if (__any_sync(kFull, sw)) {
+                    const int fb = (v >> 16) & 0xFF;
                     const int xj = S::pos(tj, kj);
-                    const uint8_t *Fb = sm + S::oF + fb * S::DS;
-                    const uint8_t *Dj = sm + S::oD + xj * S::DS;
-                    const float rs = sR[fb], cs = sC[xj], hs = sH[xj];
-                    const float dq = 0.5f * dr[xj] * (float)Frow[fb];  // D_ij F_ab
+                    const uint32_t aFj = base32 + S::oF + fb * S::DS, aDj = base32 + S::oD + xj * S::DS;
+                    const float rs = lds_f32(aR + 4 * fb), cs = lds_f32(aC + 4 * xj), hs = lds_f32(aH + 4 * xj);
+                    const float dq = 0.5f * lds_f32(aDr + 4 * xj) * (float)lds_u8(aFi + fb);  // D_ij F_ab
                     // h[m] += (D_im - D_jm) (F_b,p(m) - F_a,p(m))
                     float2 hn[K / 2 + 1];
 #pragma unroll
                     for (int k = 0; k + 1 < K; k += 2) {
-                        const uint32_t dj = *reinterpret_cast<const uint16_t *>(Dj + k * LPR + 2 * t);
+                        uint32_t dj;
+                        asm volatile("ld.shared.u16 %0, [%1];" : "=r"(dj) : "r"(aDj + k * LPR + 2 * t));
                         // 2^-25 + D_jm units
-                        const float2 mj = make_float2(__int_as_float(__byte_perm(dj, 0x33000000u, 0x7540)),
-                                                      __int_as_float(__byte_perm(dj, 0x33000000u, 0x7541)));
-                        const float2 u = sub2(fma2(make_float2(di[k], di[k + 1]), two(0.5f), two(kMmOne)), mj);
-                        const float2 v = sub2(make_float2(__int_as_float(0x4B000000 | (int)Fb[byte8(p8, k)]),
-                                                          __int_as_float(0x4B000000 | (int)Fb[byte8(p8, k + 1)])),
-                                              make_float2(mq[k], mq[k + 1]));
-                        hn[k / 2] = fma2(u, v, make_float2(hk[k], hk[k + 1]));
+                        const float2 mj = make_float2(__int_as_float((int)__byte_perm(dj, 0x33000000u, 0x7540)),
+                                                      __int_as_float((int)__byte_perm(dj, 0x33000000u, 0x7541)));
+                        const float2 u = sub2(fma2(lds_f64(aDr + 4 * k * LPR + 8 * t), two(0.5f), two(kMmOne)), mj);
+                        const float2 vv = sub2(make_float2(__int_as_float(0x4B000000 | lds_u8(entry<S>(aFj, p8, k))),
+                                                           __int_as_float(0x4B000000 | lds_u8(entry<S>(aFj, p8, k + 1)))),
+                                               make_float2(mq[k], mq[k + 1]));
+                        hn[k / 2] = fma2(u, vv, make_float2(hk[k], hk[k + 1]));
                     }
                     if constexpr (K & 1) {
                         constexpr int k = K - 1;
-                        const float mj = __int_as_float(0x33000000 | (int)Dj[k * LPR + t]);
-                        const float v = __int_as_float(0x4B000000 | (int)Fb[byte8(p8, k)]) - mq[k];
-                        hn[K / 2].x = fmaf(fmaf(di[k], 0.5f, kMmOne) - mj, v, hk[k]);
+                        const float mj = __int_as_float(0x33000000 | lds_u8(aDj + k * LPR + t));
+                        const float vv = __int_as_float(0x4B000000 | lds_u8(entry<S>(aFj, p8, k))) - mq[k];
+                        hn[K / 2].x = fmaf(fmaf(lds_f32(aDr + 4 * (k * LPR + t)), 0.5f, kMmOne) - mj, vv, hk[k]);
                     }
                     __syncwarp();  // reads of h and p by the replica's threads done
                     if (sw) {
@@ -562,13 +601,16 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
                     __syncwarp();
                     if (live && E < bestE) {
                         bestE = E;
-                        bsweep = s;
                         const uint2 b8 = *reinterpret_cast<const uint2 *>(pb + 8 * t);
 #pragma unroll
                         for (int k = 0; k < K; ++k)
                             if (t * K + k < n) gbp[t * K + k] = byte8(b8, k);
-                        if (t == 0) note_target(a, bestE, s, reached);
+                        if (t == 0) {
+                            a.best_sweep[r] = s;
+                            note_target(a, bestE, s, reached);
+                        }
                     }
+                    __syncwarp();
                 }
             }
             par ^= 1;
@@ -577,13 +619,14 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
                 ++ti;
             }
         }
-        acc_moves += moves;
+        if (live && t == 0) atomicAdd(reinterpret_cast<unsigned long long *>(a.accepted + r), (unsigned long long)moves);
     }
 
-    // ---- audit (the last unit of a call): Eq. 1 of the final permutation
-    // equals the tracked energy; write back
+    // ---- audit (the last unit of a call; a resumed unit begins with the same
+    // check): Eq. 1 of the final permutation equals the tracked energy; write
+    // back
     if (warp_live) {
-        if (part >= a.segments - 1) {
+        if (a.audit && part >= a.segments - 1) {
             int h[K], eq1 = 0;
             mm_diagonal<S>(sm, pb, n, t, h);
 #pragma unroll
@@ -596,8 +639,6 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
             if (t == 0) {
                 a.energy[r] = E;
                 a.best_energy[r] = bestE;
-                a.best_sweep[r] = bsweep;
-                a.accepted[r] = acc_moves;
             }
         }
     }
@@ -608,7 +649,7 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
 // dot_kernel for why the wait for the part before ends.
 template <class S>
 __global__ void __launch_bounds__(S::T, S::LPR == 16 ? 2 : 1) mm_kernel(const SweepArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
+    extern __shared__ __align__(1024) unsigned char smem[];
     uint32_t A[S::JT][S::REGS ? S::MT : 1][4];
     mm_stage<S>(a.D, a.F, a.n, smem, A);
     volatile int *x = reinterpret_cast<volatile int *>(smem + S::oX);
@@ -635,48 +676,125 @@ __global__ void __launch_bounds__(S::T, S::LPR == 16 ? 2 : 1) mm_kernel(const Sw
     }
 }
 
-template <int K, int LPR>
-static int mm_one(const SweepArgs &a, int grid, cudaStream_t st, MmInfo *info) {
-    using S = MmShape<K, LPR>;
-    auto fn = mm_kernel<S>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, S::bytes);
-    if (e != cudaSuccess) return (int)e;
-    if (info) {
-        info->threads = S::T;
-        info->slots = S::R;
-        info->lanes = LPR;
-        info->k = K;
-        info->smem = S::bytes;
-        return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(&info->blocks_per_sm, fn, S::T, S::bytes);
+// Persistent multi-instance kernel: CTAs take (instance, block of replicas)
+// units from `queue` and restage the tables when they move to another
+// instance. Every instance of a launch shares the compiled shape.
+template <class S>
+__global__ void __launch_bounds__(S::T, S::LPR == 16 ? 2 : 1)
+    mm_batch_kernel(const SweepArgs *__restrict__ descs, const BatchUnit *__restrict__ units, int nunits, int *queue) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ SweepArgs sa;
+    __shared__ int s_unit;
+    uint32_t A[S::JT][S::REGS ? S::MT : 1][4];
+    int cur = -1;
+    for (;;) {
+        if (threadIdx.x == 0) s_unit = atomicAdd(queue, 1);
+        __syncthreads();
+        const int u = s_unit;
+        if (u >= nunits) break;
+        const BatchUnit bu = units[u];
+        if (bu.inst != cur) {
+            const int *src = reinterpret_cast<const int *>(descs + bu.inst);
+            int *dst = reinterpret_cast<int *>(&sa);
+            for (int w = threadIdx.x; w < (int)(sizeof(SweepArgs) / sizeof(int)); w += S::T) dst[w] = src[w];
+            mm_stage<S>(descs[bu.inst].D, descs[bu.inst].F, descs[bu.inst].n, smem, A);
+            cur = bu.inst;
+        }
+        __syncthreads();
+        mm_run_block<S>(sa, bu.r0, 0, smem, A);
+        __syncthreads();
     }
-    fn<<<grid, S::T, S::bytes, st>>>(a);
+}
+
+// One launch, a query of the single-instance kernel's shape, or the
+// occupancy of the multi-instance kernel.
+struct MmCall {
+    const SweepArgs *args = nullptr;   // launch the single-instance kernel
+    const SweepArgs *descs = nullptr;  // launch the multi-instance kernel
+    const BatchUnit *units = nullptr;
+    int nunits = 0;
+    int *queue = nullptr;
+    int grid = 0;
+    cudaStream_t st = nullptr;
+    MmInfo *info = nullptr;
+    int *batch_blocks = nullptr;
+};
+
+template <int K, int LPR>
+static int mm_one(const MmCall &c) {
+    using S = MmShape<K, LPR>;
+    const bool batch = c.descs || c.batch_blocks;
+    const cudaError_t e =
+        batch ? cudaFuncSetAttribute(mm_batch_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::bytes)
+              : cudaFuncSetAttribute(mm_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::bytes);
+    if (e != cudaSuccess) return (int)e;
+    if (c.batch_blocks)
+        return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(c.batch_blocks, mm_batch_kernel<S>, S::T, S::bytes);
+    if (c.info) {
+        c.info->threads = S::T;
+        c.info->slots = S::R;
+        c.info->lanes = LPR;
+        c.info->k = K;
+        c.info->smem = S::bytes;
+        return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c.info->blocks_per_sm, mm_kernel<S>, S::T, S::bytes);
+    }
+    if (batch)
+        mm_batch_kernel<S><<<c.grid, S::T, S::bytes, c.st>>>(c.descs, c.units, c.nunits, c.queue);
+    else
+        mm_kernel<S><<<c.grid, S::T, S::bytes, c.st>>>(*c.args);
     return (int)cudaGetLastError();
 }
 
-static int mm_dispatch(int n, const SweepArgs &a, int grid, cudaStream_t st, MmInfo *info) {
+static int mm_dispatch(int n, const MmCall &c) {
+    if (n <= 32 || n > 256) return (int)cudaErrorInvalidValue;
     if (n <= 128) {
         switch ((n + 15) / 16) {
-        case 1: return mm_one<1, 16>(a, grid, st, info);
-        case 2: return mm_one<2, 16>(a, grid, st, info);
-        case 3: return mm_one<3, 16>(a, grid, st, info);
-        case 4: return mm_one<4, 16>(a, grid, st, info);
-        case 5: return mm_one<5, 16>(a, grid, st, info);
-        case 6: return mm_one<6, 16>(a, grid, st, info);
-        case 7: return mm_one<7, 16>(a, grid, st, info);
-        default: return mm_one<8, 16>(a, grid, st, info);
+        case 3: return mm_one<3, 16>(c);
+        case 4: return mm_one<4, 16>(c);
+        case 5: return mm_one<5, 16>(c);
+        case 6: return mm_one<6, 16>(c);
+        case 7: return mm_one<7, 16>(c);
+        default: return mm_one<8, 16>(c);
         }
     }
     switch ((n + 31) / 32) {
-    case 5: return mm_one<5, 32>(a, grid, st, info);
-    case 6: return mm_one<6, 32>(a, grid, st, info);
-    case 7: return mm_one<7, 32>(a, grid, st, info);
-    case 8: return mm_one<8, 32>(a, grid, st, info);
-    default: return (int)cudaErrorInvalidValue;
+    case 5: return mm_one<5, 32>(c);
+    case 6: return mm_one<6, 32>(c);
+    case 7: return mm_one<7, 32>(c);
+    default: return mm_one<8, 32>(c);
     }
 }
 
-int mm_query(int n, MmInfo *info) { return mm_dispatch(n, SweepArgs{}, 0, nullptr, info); }
+int mm_query(int n, MmInfo *info) {
+    MmCall c;
+    c.info = info;
+    return mm_dispatch(n, c);
+}
 
-int mm_launch(const SweepArgs &a, int grid, cudaStream_t st) { return mm_dispatch(a.n, a, grid, st, nullptr); }
+int mm_launch(const SweepArgs &a, int grid, cudaStream_t st) {
+    MmCall c;
+    c.args = &a;
+    c.grid = grid;
+    c.st = st;
+    return mm_dispatch(a.n, c);
+}
+
+int mm_batch_blocks_per_sm(int n, int *blocks) {
+    MmCall c;
+    c.batch_blocks = blocks;
+    return mm_dispatch(n, c);
+}
+
+int mm_batch_launch(int n, const SweepArgs *descs, const BatchUnit *units, int nunits, int *queue, int grid,
+                    cudaStream_t st) {
+    MmCall c;
+    c.descs = descs;
+    c.units = units;
+    c.nunits = nunits;
+    c.queue = queue;
+    c.grid = grid;
+    c.st = st;
+    return mm_dispatch(n, c);
+}
 
 }  // namespace pdit

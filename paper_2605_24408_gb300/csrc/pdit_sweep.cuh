@@ -69,6 +69,7 @@ struct SweepArgs {
     int fresh;             // start from a Fisher-Yates permutation
     int table_in;          // take the influence table from `tables` instead of rebuilding it
     int table_out;         // leave the influence table in `tables` at the end
+    int audit;             // tensor-core product kernel: check the final energies against Eq. 1
     // per-replica state, indexed by local replica id
     int32_t *perm;
     int32_t *best_perm;
@@ -1742,5 +1743,8 @@ struct MmInfo {
 };
 int mm_query(int n, MmInfo *info);
 int mm_launch(const SweepArgs &a, int grid, cudaStream_t stream);
+int mm_batch_blocks_per_sm(int n, int *blocks);
+int mm_batch_launch(int n, const SweepArgs *descs, const BatchUnit *units, int nunits, int *queue, int grid,
+                    cudaStream_t stream);
 
 }  // namespace pdit
