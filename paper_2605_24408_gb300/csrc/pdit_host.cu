@@ -97,6 +97,7 @@ struct Plan {
     bool tsmem = true, cls = false, dot = false;
     bool mm = false;  // with dot: the tensor-core product kernel (pdit_mma.cu)
     int lanes = 32;   // its threads per replica
+    bool small = false;  // the small kernel (pdit_small.cu)
     int stride = 0, sv_len = 0, cupim_off = 0, v2_off = 0, rc_off = 0, dstride = 0;
     size_t table_elems = 0;  // int32 entries of one replica's saved table (workspace)
     size_t df_bytes = 0, group_bytes = 0, smem = 0;
@@ -419,6 +420,35 @@ int auto_dot_plan(const pdit_qap *h, int replicas, Plan *p, size_t reserve) {
     return make_dot_plan(h, replicas, h->force_wpr, p, reserve);
 }
 
+// Launch shape of the small kernel: one warp per replica, a call's replicas
+// spread over the SMs first, then up to 16 to a CTA.
+int make_small_plan(const pdit_qap *h, int replicas, Plan *p) {
+    const int most = h->force_groups > 0 ? std::min(16, h->force_groups) : 16;
+    const int per_sm = (replicas + h->num_sms - 1) / h->num_sms;
+    p->small = true;
+    p->tsmem = true;
+    p->pk = p->wpr = p->maxk = 1;
+    p->table_elems = 0;
+    p->groups = std::max(1, std::min(most, per_sm));
+    p->threads = 32 * p->groups;
+    pdit::SmallInfo info{};
+    const int e = pdit::small_query(h->n, p->groups, &info);
+    if (e != 0) return cuda_fail((cudaError_t)e, "occupancy query");
+    if (info.blocks_per_sm < 1 || info.smem > h->smem_optin) return PDIT_ENOTSUP;
+    p->smem = info.smem;
+    const int need = (replicas + p->groups - 1) / p->groups;
+    p->grid = std::max(1, std::min(need, h->num_sms * info.blocks_per_sm));
+    return PDIT_OK;
+}
+
+// Whether a call runs the small kernel: at most 32 locations, symmetric, a
+// sequential mode, no table dump, and no setting that asks for another kernel
+// (dot products, pending terms, more than one warp per replica).
+bool use_small_path(const pdit_qap *h, const pdit_opts *o) {
+    return h->n <= 32 && !h->asym && o->mode != PDIT_MODE_CUPIM && !o->tables && h->force_wpr <= 1 &&
+           h->force_pk <= 1 && h->force_place != PDIT_PLACE_GLOBAL && h->force_infl != PDIT_INFLUENCE_PRODUCTS;
+}
+
 // The product kernel of a call: tensor-core products where the instance
 // allows them and no wider mapping than a warp per replica is asked for, else
 // the dot-product kernel. `any`: also where the automatic rule prefers the
@@ -444,6 +474,11 @@ bool use_dot_path(const pdit_qap *h, const pdit_opts *o) {
 // the table kernels.
 int plan_for(const pdit_qap *h, const pdit_opts *o, Plan *p) {
     if (use_class_path(h, o)) return make_class_plan(h, o->replicas, h->force_wpr, p);
+    if (use_small_path(h, o)) {
+        const int rc = make_small_plan(h, o->replicas, p);
+        if (rc != PDIT_ENOTSUP) return rc;
+        *p = Plan();
+    }
     if (h->force_infl == PDIT_INFLUENCE_PRODUCTS) {
         if (!dot_eligible(h) || o->mode == PDIT_MODE_CUPIM || o->tables) return PDIT_ENOTSUP;
         return product_plan(h, o->replicas, p, 0, true);
@@ -521,7 +556,7 @@ int parts_of(const pdit_opts *o, const Plan &p, int span) {
 // kept between calls by the server, the dot kernel's permuted flow matrix;
 // either kernel's table between the parts of a launch).
 bool needs_tables(const pdit_opts *o, const Plan &p, bool persist = false, bool whole = false) {
-    if (p.mm) return false;  // its state is the permutation and the energies
+    if (p.mm || p.small) return false;  // their state is the permutation and the energies
     return persist || o->mode == PDIT_MODE_PT || (!p.dot && !p.tsmem) || (!whole && may_split(o, p));
 }
 
@@ -1042,6 +1077,7 @@ int pdit_anneal_ex(pdit_qap *h, const pdit_opts *o) {
             PDIT_CK(cudaMemsetAsync(w.queue, 0, sizeof(int32_t), st));
             if (a.segments > 1) PDIT_CK(cudaMemsetAsync(w.seg_done, 0, sizeof(int32_t) * R, st));
             const int e = plan.cls ? class_launch(h->dt_bytes, plan, a, st)
+                        : plan.small ? pdit::small_launch(a, plan.grid, plan.groups, st)
                         : plan.mm  ? pdit::mm_launch(a, plan.grid, st)
                         : plan.dot ? pdit::dot_launch(plan.maxk, plan.wpr, a, plan.grid, plan.threads, plan.smem, st)
                                    : sweep_launch(h->dt_bytes, h->asym != 0, plan, a, st);

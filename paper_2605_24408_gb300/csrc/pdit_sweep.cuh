@@ -1734,6 +1734,15 @@ int dot_batch_blocks_per_sm(int maxk, int wpr, int threads, size_t smem, int *bl
 int dot_batch_launch(int maxk, int wpr, const SweepArgs *descs, const BatchUnit *units, int nunits, int *queue,
                      int grid, int threads, size_t smem, cudaStream_t stream);
 
+// Small kernel (pdit_small.cu): symmetric instances of at most 32 locations,
+// one warp per replica. Return a cudaError_t value.
+struct SmallInfo {
+    int blocks_per_sm;
+    size_t smem;
+};
+int small_query(int n, int warps, SmallInfo *info);
+int small_launch(const SweepArgs &a, int grid, int warps, cudaStream_t stream);
+
 // Tensor-core product kernel (pdit_mma.cu): symmetric instances with zero
 // diagonals and entries in 0..127; one compiled kernel per range of n.
 // Return a cudaError_t value.
