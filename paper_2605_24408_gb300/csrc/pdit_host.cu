@@ -28,6 +28,7 @@ struct pdit_qap {
     int cls_f = 0;
     long long cls_e0 = 0;
     uint8_t *dx = nullptr;  // x_c on the device
+    int f32_ok = 0;         // 8 (n + 2) max|D| max|F| < 2^24: every entry and energy exact in binary32
     int nonneg = 0;         // every entry of D and F >= 0
     int packed_ok = 0;      // max-min of D and of F <= 127: swap factors fit int8
     std::vector<int32_t> hD, hF;
@@ -432,7 +433,7 @@ int make_small_plan(const pdit_qap *h, int replicas, Plan *p) {
     p->groups = std::max(1, std::min(most, per_sm));
     p->threads = 32 * p->groups;
     pdit::SmallInfo info{};
-    const int e = pdit::small_query(h->n, p->groups, &info);
+    const int e = pdit::small_query(h->n, h->f32_ok != 0, p->groups, &info);
     if (e != 0) return cuda_fail((cudaError_t)e, "occupancy query");
     if (info.blocks_per_sm < 1 || info.smem > h->smem_optin) return PDIT_ENOTSUP;
     p->smem = info.smem;
@@ -848,6 +849,7 @@ int qap_prepare(int n, const int32_t *D, const int32_t *F, pdit_qap **out) {
         h->cls_f = (int)fcls;
         h->cls_e0 = f0 * dsum;  // D's diagonal is zero
     }
+    h->f32_ok = (int64_t)8 * (n + 2) * maxd * maxf < ((int64_t)1 << 24) ? 1 : 0;
     h->nonneg = dlo >= 0 && flo >= 0 ? 1 : 0;
     h->packed_ok = (dhi - dlo <= 127 && fhi - flo <= 127) ? 1 : 0;
     const int64_t mx = std::max(maxd, maxf);
@@ -1077,7 +1079,7 @@ int pdit_anneal_ex(pdit_qap *h, const pdit_opts *o) {
             PDIT_CK(cudaMemsetAsync(w.queue, 0, sizeof(int32_t), st));
             if (a.segments > 1) PDIT_CK(cudaMemsetAsync(w.seg_done, 0, sizeof(int32_t) * R, st));
             const int e = plan.cls ? class_launch(h->dt_bytes, plan, a, st)
-                        : plan.small ? pdit::small_launch(a, plan.grid, plan.groups, st)
+                        : plan.small ? pdit::small_launch(a, h->f32_ok != 0, plan.grid, plan.groups, st)
                         : plan.mm  ? pdit::mm_launch(a, plan.grid, st)
                         : plan.dot ? pdit::dot_launch(plan.maxk, plan.wpr, a, plan.grid, plan.threads, plan.smem, st)
                                    : sweep_launch(h->dt_bytes, h->asym != 0, plan, a, st);

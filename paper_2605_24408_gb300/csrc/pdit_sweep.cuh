@@ -1735,13 +1735,14 @@ int dot_batch_launch(int maxk, int wpr, const SweepArgs *descs, const BatchUnit 
                      int grid, int threads, size_t smem, cudaStream_t stream);
 
 // Small kernel (pdit_small.cu): symmetric instances of at most 32 locations,
-// one warp per replica. Return a cudaError_t value.
+// one warp per replica; f32: its integers in binary32 (see that file). Return
+// a cudaError_t value.
 struct SmallInfo {
     int blocks_per_sm;
     size_t smem;
 };
-int small_query(int n, int warps, SmallInfo *info);
-int small_launch(const SweepArgs &a, int grid, int warps, cudaStream_t stream);
+int small_query(int n, bool f32, int warps, SmallInfo *info);
+int small_launch(const SweepArgs &a, bool f32, int grid, int warps, cudaStream_t stream);
 
 // Tensor-core product kernel (pdit_mma.cu): symmetric instances with zero
 // diagonals and entries in 0..127; one compiled kernel per range of n.
