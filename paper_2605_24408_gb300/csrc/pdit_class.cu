@@ -14,26 +14,75 @@
 // it G_m += D_mw - D_mu. These are Eq. 3's exact values, so every Eq. 5 draw
 // and the whole trajectory equal those of the table kernels; the N x N
 // influence table becomes the vector G and an accepted swap costs O(N).
+//
+// A group of 32 * WPR threads runs one replica; thread t owns the MAXK
+// consecutive locations t*MAXK + k and keeps their G and class bits in
+// registers, so its swap energies go to the draw in registers, in outcome
+// order, and a row of D is read as one or two wide words per thread. Shared
+// memory keeps the copies other threads read (G_i, and the facilities for
+// swaps).
+//
+// Bound: issue slots (about 190 instructions an update at N = 256 and one
+// warp per replica); 27 one-warp replicas an SM of 64 registers a thread hide
+// the chain, and 4096 replicas are one round.
 #include "pdit_sweep.cuh"
 
 namespace pdit {
 
+// MAXK consecutive entries of a row of D, from a 16-byte aligned row.
+template <typename DT, int MAXK>
+__device__ __forceinline__ void load_entries(const DT *p, int (&v)[MAXK]) {
+    constexpr int B = MAXK * (int)sizeof(DT);
+    if constexpr (B <= 2 || MAXK == 1) {
+#pragma unroll
+        for (int k = 0; k < MAXK; ++k) v[k] = p[k];
+    } else {
+        constexpr int W = B / 4;  // 32-bit words
+        uint32_t w[W];
+        if constexpr (W == 1) {
+            w[0] = *reinterpret_cast<const uint32_t *>(p);
+        } else if constexpr (W == 2) {
+            const uint2 x = *reinterpret_cast<const uint2 *>(p);
+            w[0] = x.x;
+            w[1] = x.y;
+        } else {
+#pragma unroll
+            for (int q = 0; q < W / 4; ++q) {
+                const uint4 x = reinterpret_cast<const uint4 *>(p)[q];
+                w[4 * q] = x.x;
+                w[4 * q + 1] = x.y;
+                w[4 * q + 2] = x.z;
+                w[4 * q + 3] = x.w;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < MAXK; ++k) {
+            if constexpr (sizeof(DT) == 1)
+                v[k] = (int)(int8_t)(w[k / 4] >> (8 * (k & 3)));
+            else if constexpr (sizeof(DT) == 2)
+                v[k] = (int)(int16_t)(w[k / 2] >> (16 * (k & 1)));
+            else
+                v[k] = (int)w[k];
+        }
+    }
+}
+
 template <typename DT, int MAXK, int WPR>
 __device__ __forceinline__ void run_class_replica(const SweepArgs &a, int r, int t, int bar, const DT *sD,
-                                                  const uint8_t *sx, int32_t *sp, int32_t *sG, int32_t *sv,
-                                                  GroupScratch *gs) {
+                                                  const uint8_t *sx, int32_t *sp, int32_t *sG, GroupScratch *gs) {
     constexpr int G = 32 * WPR;
     const int lane = t & 31;
     const int wg = t >> 5;
     const int n = a.n;
     const int npad = (n + 3) & ~3;
+    const int ds = a.dstride;  // row stride of D (entries): whole 16-byte words
     const uint32_t grep = a.rep_base + (uint32_t)r;
     int32_t *gp = a.perm + (size_t)r * n;
     int32_t *gbp = a.best_perm + (size_t)r * n;
     const int f2 = 2 * a.cls_f;
 
     if (a.fresh) {
-        fisher_yates<WPR>(a, grep, n, t, sv, sp, bar);
+        fisher_yates<WPR>(a, grep, n, t, sG, sp, bar);
     } else {
         for (int m = t; m < n; m += G) sp[m] = gp[m];
     }
@@ -44,7 +93,7 @@ __device__ __forceinline__ void run_class_replica(const SweepArgs &a, int r, int
         for (int m = t; m < n; m += G) sG[m] = a.tables[(size_t)r * npad + m];
     } else {
         for (int m = t; m < n; m += G) {
-            const DT *Dm = sD + m * n;
+            const DT *Dm = sD + m * ds;
             int acc = 0;
             for (int j = 0; j < n; ++j) acc += sx[sp[j]] ? (int)Dm[j] : 0;
             sG[m] = acc;
@@ -87,15 +136,15 @@ __device__ __forceinline__ void run_class_replica(const SweepArgs &a, int r, int
     const float beta_fixed = a.sweep_end <= a.sweep_begin ? 0.0f
                            : a.mode == 1 ? a.beta[a.rung[r]] : a.mode == 2 ? a.beta[r] : 0.0f;
 
-    // Each thread keeps, for its candidates j = t + G k, the class bit of the
-    // facility at j and G_j in registers; it also applies the G update for
-    // exactly these j, so they stay equal to shared memory, which keeps the
-    // copies other threads read (G_i at the start of every update).
-    int cx[MAXK], cg[MAXK];
+    // this thread's locations: class bits of their facilities (bit k) and G
+    const int j0 = t * MAXK;
+    const int jr = j0 < n ? j0 : 0;  // threads beyond n read the row's start
+    unsigned cx = 0;
+    int cg[MAXK];
 #pragma unroll
     for (int k = 0; k < MAXK; ++k) {
-        const int j = t + G * k;
-        cx[k] = j < n ? sx[sp[j]] : 0;
+        const int j = j0 + k;
+        cx |= (j < n ? (unsigned)sx[sp[j]] : 0u) << k;
         cg[k] = j < n ? sG[j] : 0;
     }
 
@@ -114,53 +163,37 @@ __device__ __forceinline__ void run_class_replica(const SweepArgs &a, int r, int
             for (int ii = 0; ii < cnt; ++ii) {
                 const int i = i0 + ii;
                 const uint32_t draw_hi = __shfl_sync(kFull, rw.y, ii);
-                const int xa = sx[sp[i]];
+                const int fa = sp[i];
+                const int xa = sx[fa];
                 const int gi = sG[i];
-                const DT *Di = sD + i * n;
                 // ---- swap energies: 0 within a class, 2 f (G_w - G_u - D_uw) across
-                int dself = 0;  // MAXK = 1: this thread's energy, handed to the draw in a register
+                int di[MAXK], dc[MAXK];
+                load_entries<DT, MAXK>(sD + i * ds + jr, di);
+                const int sgn = xa ? f2 : -f2;
+                const unsigned differ = xa ? ~cx : cx;
 #pragma unroll
                 for (int k = 0; k < MAXK; ++k) {
-                    const int j = t + G * k;
-                    if (j < n) {
-                        int d = 0;
-                        if (cx[k] != xa) {
-                            const int gd = cg[k] - gi;
-                            d = f2 * ((xa ? gd : -gd) - (int)Di[j]);
-                        }
-                        if constexpr (MAXK > 1)
-                            sv[j] = d;
-                        else
-                            dself = d;
-                    }
+                    const int d = sgn * (cg[k] - gi) - f2 * di[k];
+                    dc[k] = differ & (1u << k) ? d : 0;
                 }
-                const int3 sel = eq5_draw<MAXK, WPR>(
-                    sv, sp, n, t, dself, MAXK == 1 && t < n ? sp[t] : 0, beta, draw_hi,
+                const int3 sel = eq5_draw_regs<MAXK, WPR>(
+                    dc, [&](int kk) { return sp[j0 + kk]; }, n, t, beta, draw_hi,
                     [&]() { return __shfl_sync(kFull, rw.x, ii); }, draw_tag(i, s), bar, gs);
                 const int js = sel.x, dstar = sel.y, fb = sel.z;
                 if (js == i) continue;
-                const int fa = sp[i];
                 const int xb = sx[fb];
-                // ---- apply: G moves only when the classes differ
+                // ---- apply: G and the class bits move only when the classes differ
                 if (xb != xa) {
-                    const DT *Dj = sD + js * n;
+                    int dj[MAXK];
+                    load_entries<DT, MAXK>(sD + js * ds + jr, dj);
 #pragma unroll
                     for (int k = 0; k < MAXK; ++k) {
-                        const int m = t + G * k;
-                        if (m < n) {
-                            const int dd = (int)Dj[m] - (int)Di[m];
-                            const int v = xa ? dd : -dd;
-                            sG[m] += v;
-                            cg[k] += v;
-                        }
+                        const int v = dj[k] - di[k];
+                        cg[k] += xa ? v : -v;
+                        if (j0 + k < n) sG[j0 + k] = cg[k];
                     }
-                }
-                // the facilities at i and js moved
-#pragma unroll
-                for (int k = 0; k < MAXK; ++k) {
-                    const int j = t + G * k;
-                    if (j == i) cx[k] = xb;
-                    if (j == js) cx[k] = xa;
+                    if ((unsigned)(i - j0) < (unsigned)MAXK) cx ^= 1u << (i - j0);
+                    if ((unsigned)(js - j0) < (unsigned)MAXK) cx ^= 1u << (js - j0);
                 }
                 E += dstar;
                 acc_moves += 1;
@@ -182,7 +215,7 @@ __device__ __forceinline__ void run_class_replica(const SweepArgs &a, int r, int
 
     // ---- audit: G recomputed from the final permutation equals the tracked one
     for (int m = t; m < n; m += G) {
-        const DT *Dm = sD + m * n;
+        const DT *Dm = sD + m * ds;
         int acc = 0;
         for (int j = 0; j < n; ++j) acc += sx[sp[j]] ? (int)Dm[j] : 0;
         if (acc != sG[m]) atomicOr(a.status, 1);
@@ -202,8 +235,8 @@ __device__ __forceinline__ void run_class_replica(const SweepArgs &a, int r, int
 }
 
 // Persistent: each group of 32 * WPR threads pulls replicas from a.queue.
-// Shared memory: D as DT (n x n), x of every facility (bytes, padded to 16),
-// then per group: scratch, p, G, and the scratch vector of swap energies.
+// Shared memory: D as DT (n rows of 16-byte words), x of every facility
+// (bytes, padded to 16), then per group: scratch, p and G.
 template <typename DT, int MAXK, int WPR>
 __global__ void __launch_bounds__(class_bound(MAXK, WPR)) class_kernel(const SweepArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -214,21 +247,23 @@ __global__ void __launch_bounds__(class_bound(MAXK, WPR)) class_kernel(const Swe
     const int t = threadIdx.x % G;
     const int bar = 1 + grp;
     DT *sD = reinterpret_cast<DT *>(smem);
-    uint8_t *sx = smem + (((size_t)n * n * sizeof(DT) + 15) & ~(size_t)15);
-    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) sD[idx] = static_cast<DT>(a.D[idx]);
+    uint8_t *sx = smem + (size_t)n * a.dstride * sizeof(DT);
+    for (int idx = threadIdx.x; idx < n * a.dstride; idx += blockDim.x) {
+        const int m = idx / a.dstride, c = idx - m * a.dstride;
+        sD[idx] = c < n ? static_cast<DT>(a.D[m * n + c]) : (DT)0;
+    }
     for (int c = threadIdx.x; c < n; c += blockDim.x) sx[c] = a.cls_x[c];
     __syncthreads();
     unsigned char *gb = smem + a.df_bytes + (size_t)grp * a.group_bytes;
     GroupScratch *gs = reinterpret_cast<GroupScratch *>(gb);
     int32_t *sp = reinterpret_cast<int32_t *>(gb + kScratchBytes);
     int32_t *sG = sp + npad;
-    int32_t *sv = sG + npad;
     for (;;) {
         if (t == 0) gs->item = atomicAdd(a.queue, 1);
         group_sync<WPR>(bar);
         const int item = gs->item;
         if (item >= a.replicas) break;
-        run_class_replica<DT, MAXK, WPR>(a, item, t, bar, sD, sx, sp, sG, sv, gs);
+        run_class_replica<DT, MAXK, WPR>(a, item, t, bar, sD, sx, sp, sG, gs);
     }
 }
 

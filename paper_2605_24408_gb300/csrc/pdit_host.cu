@@ -258,10 +258,11 @@ int make_class_plan(const pdit_qap *h, int replicas, int wpr, Plan *p) {
     p->pk = 1;
     p->stride = npad;
     p->table_elems = (size_t)npad;  // G
-    p->sv_len = cover;
-    p->dstride = n;
-    p->df_bytes = align_up((size_t)n * n * h->dt_bytes, 16) + align_up((size_t)npad, 16);
-    p->group_bytes = align_up(pdit::kScratchBytes + (size_t)4 * (2 * npad + cover), 16);
+    p->sv_len = 0;
+    // rows of D: whole 16-byte words, and whole groups of a thread's candidates
+    p->dstride = (int)align_up((size_t)n, std::max<size_t>(16 / h->dt_bytes, 8));
+    p->df_bytes = (size_t)n * p->dstride * h->dt_bytes + align_up((size_t)npad, 16);
+    p->group_bytes = align_up(pdit::kScratchBytes + (size_t)4 * (2 * npad), 16);
     const size_t budget = h->smem_optin;
     if (p->df_bytes + p->group_bytes > budget) return PDIT_ENOTSUP;
     const int fit = (int)((budget - p->df_bytes) / p->group_bytes);

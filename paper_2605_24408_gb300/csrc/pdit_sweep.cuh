@@ -1717,7 +1717,7 @@ int class_blocks_per_sm(int maxk, int wpr, int threads, size_t smem, int *blocks
 template <typename DT>
 int class_launch(int maxk, int wpr, const SweepArgs &a, int grid, int threads, size_t smem, cudaStream_t stream);
 __host__ __device__ constexpr int class_bound(int maxk, int wpr) {
-    return maxk >= 4 ? 512 : 1024;
+    return maxk == 8 ? 896 : 1024;  // eight candidates a thread: 72 registers
 }
 
 // Dot-product sweep kernels (pdit_dot.cu): symmetric instances with every
