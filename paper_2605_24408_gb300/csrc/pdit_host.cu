@@ -368,16 +368,20 @@ int make_dot_plan(const pdit_qap *h, int replicas, int wpr, Plan *p, size_t rese
     return PDIT_OK;
 }
 
-// Whether an instance can run the tensor-core product kernel: symmetric, zero
-// diagonals, every entry of D and F in 0..127.
-bool mm_eligible(const pdit_qap *h) { return !h->asym && h->zero_diag && h->dt_bytes == 1 && h->nonneg; }
+// Whether an instance can run the tensor-core product kernel: zero diagonals
+// and every entry of D and F in 0..127; the general form also with every
+// energy below 2^24 and up to the sizes whose four tables fit.
+bool mm_eligible(const pdit_qap *h) {
+    if (!h->zero_diag || h->dt_bytes != 1 || !h->nonneg || h->n <= 32) return false;
+    return !h->asym || (h->f32_ok && h->n <= pdit::kMmGeneralMax);
+}
 
 // Launch shape of the tensor-core product kernel: its thread mapping and
 // shared memory are fixed by n (MmInfo); replicas per CTA spread the call
 // over the GPU.
 int make_mm_plan(const pdit_qap *h, int replicas, Plan *p, size_t reserve = 0) {
     pdit::MmInfo info{};
-    const int e = pdit::mm_query(h->n, &info);
+    const int e = pdit::mm_query(h->n, h->asym != 0, &info);
     if (e != 0) return cuda_fail((cudaError_t)e, "occupancy query");
     if (info.blocks_per_sm < 1 || info.smem + reserve > h->smem_optin) return PDIT_ENOTSUP;
     p->dot = p->mm = true;
@@ -456,19 +460,21 @@ bool use_small_path(const pdit_qap *h, const pdit_opts *o) {
 // the dot-product kernel. `any`: also where the automatic rule prefers the
 // table kernels.
 int product_plan(const pdit_qap *h, int replicas, Plan *p, size_t reserve, bool any) {
-    if (mm_eligible(h) && h->force_wpr <= 1 && h->n > 32) {
+    if (mm_eligible(h) && h->force_wpr <= 1) {
         const int rc = make_mm_plan(h, replicas, p, reserve);
         if (rc != PDIT_ENOTSUP) return rc;
         *p = Plan();
     }
+    if (h->asym) return PDIT_ENOTSUP;
     return any ? make_dot_plan(h, replicas, h->force_wpr, p, reserve) : auto_dot_plan(h, replicas, p, reserve);
 }
 
-// Whether a call runs the dot-product kernel: an eligible instance in a
-// sequential mode, without a request for the table dump or for table-kernel
+// Whether a call runs a product kernel by the automatic choice: an eligible
+// instance in a sequential mode, without a request for the table dump or for table-kernel
 // knobs (pending terms, table placement), unless the handle asks for it.
 bool use_dot_path(const pdit_qap *h, const pdit_opts *o) {
-    if (!dot_eligible(h) || o->mode == PDIT_MODE_CUPIM || o->tables) return false;
+    if (!dot_eligible(h) && !mm_eligible(h)) return false;
+    if (o->mode == PDIT_MODE_CUPIM || o->tables) return false;
     return h->force_infl == PDIT_INFLUENCE_AUTO && h->force_pk == 0 && h->force_place == PDIT_PLACE_AUTO;
 }
 
@@ -1081,7 +1087,7 @@ int pdit_anneal_ex(pdit_qap *h, const pdit_opts *o) {
             if (a.segments > 1) PDIT_CK(cudaMemsetAsync(w.seg_done, 0, sizeof(int32_t) * R, st));
             const int e = plan.cls ? class_launch(h->dt_bytes, plan, a, st)
                         : plan.small ? pdit::small_launch(a, h->f32_ok != 0, plan.grid, plan.groups, st)
-                        : plan.mm  ? pdit::mm_launch(a, plan.grid, st)
+                        : plan.mm  ? pdit::mm_launch(a, h->asym != 0, plan.grid, st)
                         : plan.dot ? pdit::dot_launch(plan.maxk, plan.wpr, a, plan.grid, plan.threads, plan.smem, st)
                                    : sweep_launch(h->dt_bytes, h->asym != 0, plan, a, st);
             if (e != 0) return cuda_fail((cudaError_t)e, "sweep kernel launch");
@@ -1545,7 +1551,7 @@ int batch_blocks_t(const BatchClass &c, int *blocks) {
 }
 
 int batch_blocks(const BatchClass &c, int *blocks) {
-    if (c.mm) return pdit::mm_batch_blocks_per_sm(c.n, blocks);
+    if (c.mm) return pdit::mm_batch_blocks_per_sm(c.n, c.asym, blocks);
     if (c.dot) return pdit::dot_batch_blocks_per_sm(c.maxk, c.wpr, c.threads, c.smem, blocks);
     return c.asym ? batch_blocks_t<true>(c, blocks) : batch_blocks_t<false>(c, blocks);
 }
@@ -1563,7 +1569,7 @@ int batch_launch_t(const BatchClass &c, const pdit::SweepArgs *descs, int *queue
 }
 
 int batch_launch(const BatchClass &c, const pdit::SweepArgs *descs, int *queue) {
-    if (c.mm) return pdit::mm_batch_launch(c.n, descs, c.d_units, c.nunits, queue, c.grid, c.stream);
+    if (c.mm) return pdit::mm_batch_launch(c.n, c.asym, descs, c.d_units, c.nunits, queue, c.grid, c.stream);
     if (c.dot)
         return pdit::dot_batch_launch(c.maxk, c.wpr, descs, c.d_units, c.nunits, queue, c.grid, c.threads, c.smem,
                                       c.stream);
@@ -1572,7 +1578,7 @@ int batch_launch(const BatchClass &c, const pdit::SweepArgs *descs, int *queue) 
 
 // Same compiled kernel shape.
 bool same_class(const BatchClass &x, int dt, bool asym, const Plan &p) {
-    if (x.mm || p.mm) return x.mm == p.mm && x.maxk == p.maxk && x.lanes == p.lanes;
+    if (x.mm || p.mm) return x.mm == p.mm && x.asym == asym && x.maxk == p.maxk && x.lanes == p.lanes;
     if (x.dot || p.dot) return x.dot == p.dot && x.maxk == p.maxk && x.wpr == p.wpr;
     return x.dt == dt && x.asym == asym && x.maxk == p.maxk && x.wpr == p.wpr && x.pk == p.pk && x.tsmem == p.tsmem;
 }

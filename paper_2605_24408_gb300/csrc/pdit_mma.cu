@@ -26,20 +26,36 @@
 // t*K + k. Steps of one update: the gathers (each replica's threads), a CTA
 // barrier, the products (each warp holds its rows of D or F for all
 // replicas), a barrier, and energies, draw and swap (each replica's threads).
+// General instances (ASYM: D or F not symmetric) keep Eq. 2's two-term table,
+//   T[j][a]    = sum_y D[j][y] F[a][p(y)] + D[y][j] F[p(y)][a],
+//   T[i][p(j)] = sum_c F[p(j)][c] D[i][p^-1(c)] + F[c][p(j)] D[p^-1(c)][i]:
+// the same products of twice the depth, [D | D^T] and [F | F^T] against
+// [q; q'] and [g; g']. A unit of energy is then 2^-48 itself.
+//
+// Bound: the latency of an update's chain of about 450 instructions a warp
+// (issue slots 50% busy, 16 warps an SM at the register limit; shared-memory
+// pipe 60%, tensor pipe 23%). Byte permutes that form a gather's address from
+// its row's, warp-uniform control and replicas paired in warps from the first
+// took N = 100, 4096 replicas, from 2.13e9 to 2.39e9 updates/s (1.12e9 with
+// the dot-product kernel); N = 256, 2048 replicas: 7.3e8 (1.6e8 with the table
+// kernels). Bytes instead of f16 words for the vectors, with h in registers,
+// cut the wavefronts by a fifth but were slower (2.03e9: more instructions);
+// products formed one location ahead by warps of their own were too (1.78e9).
 #include "pdit_sweep.cuh"
 
 namespace pdit {
 
-template <int K_, int LPR_>
+template <int K_, int LPR_, bool ASYM_ = false>
 struct MmShape {
     static constexpr int K = K_, LPR = LPR_;
+    static constexpr bool ASYM = ASYM_;
     static constexpr int NP = K * LPR;            // padded size
     static constexpr int MT = NP / 16;            // 16-row tiles of D and of F; 16-deep steps of a product
     static constexpr int NW = LPR == 16 ? 8 : 16; // warps per CTA
     static constexpr int T = 32 * NW;
     static constexpr int R = 16;                  // replica slots per CTA
     static constexpr int JT = (MT + NW / 2 - 1) / (NW / 2);  // row tiles per warp
-    static constexpr bool REGS = MT <= 8;         // the warp's rows stay in registers
+    static constexpr bool REGS = MT <= 8 && !ASYM;         // the warp's rows stay in registers
     // Row strides. Tables, bytes: 256 where the fragments are read once, so
     // that a gather's address is its row's with the byte index for the low
     // byte (one byte permute); else 16 x odd, so that 8 rows x 16 bytes read
@@ -53,7 +69,10 @@ struct MmShape {
     static constexpr int CS = NP + 4;
     static constexpr int PS = 8 * LPR;            // permutation bytes of a replica (8 per thread)
     // shared memory (the tables first: their rows are 256-byte aligned)
-    static constexpr int oD = 0, oF = oD + NP * DS, oVq = oF + NP * DS, oVg = oVq + R * VS, oC = oVg + R * VS,
+    static constexpr int TT = NP * DS, VT = R * VS;  // from a table, a vector, to its transpose's
+    static constexpr int NT2 = ASYM ? 2 : 1;      // the transposes after D and F, their vectors after q and g
+    static constexpr int oD = 0, oF = oD + NT2 * NP * DS, oVq = oF + NT2 * NP * DS, oVg = oVq + NT2 * R * VS,
+                         oC = oVg + NT2 * R * VS,
                          oR = oC + 4 * R * CS, oH = oR + 4 * R * CS, oP = oH + 4 * R * CS, oI = oP + R * PS,
                          oDr = oI + R * PS, oX = oDr + 8 * NP, bytes = oX + 16;
     // result row of the replica in vector row v: bits 1 and 2 of v trade places
@@ -76,8 +95,8 @@ struct MmShape {
     }
 };
 
-constexpr float kMmUnit = 3.552713678800501e-15f;   // 2^-48: one unit of energy / 2
-constexpr float kMmScale = 5.62949953421312e14f;    // 2^49: energy per unit
+constexpr float kMmUnit = 3.552713678800501e-15f;   // 2^-48: half a unit of energy (general form: one)
+constexpr float kMmScale = 5.62949953421312e14f;    // 2^49: energy per 1.0 (general form: 2^48)
 constexpr float kMmOne = 2.98023223876953125e-08f;  // 2^-25: the unit in its last place
 
 // Two binary32 operations at once (each rounded as the single one).
@@ -140,8 +159,8 @@ struct MmVals {
 
 // The exact draw (eq5_draw_exact) for one replica's LPR threads.
 template <int K, int LPR>
-__device__ __noinline__ int mm_exact_draw(const MmVals<K> d, int n, int t, float beta, unsigned long long draw,
-                                          unsigned mask) {
+__device__ __noinline__ int mm_exact_draw(const MmVals<K> d, int n, int t, float scale, float beta,
+                                          unsigned long long draw, unsigned mask) {
     float dmin = __int_as_float(0x7F800000);
 #pragma unroll
     for (int k = 0; k < K; ++k)
@@ -152,7 +171,7 @@ __device__ __noinline__ int mm_exact_draw(const MmVals<K> d, int n, int t, float
     unsigned long long lsum = 0;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-        if (t * K + k < n) lsum += eq5_weight_f((d.v[k] - dmin) * kMmScale, beta);
+        if (t * K + k < n) lsum += eq5_weight_f((d.v[k] - dmin) * scale, beta);
         pre[k] = lsum;
     }
     unsigned long long incl = lsum;
@@ -209,12 +228,16 @@ template <class S>
 __device__ __forceinline__ void mm_stage(const int32_t *D, const int32_t *F, int n, unsigned char *sm,
                                          uint32_t (&A)[S::JT][S::REGS ? S::MT : 1][4]) {
     uint32_t *z = reinterpret_cast<uint32_t *>(sm + S::oD);
-    for (int w = threadIdx.x; w < 2 * S::NP * S::DS / 4; w += S::T) z[w] = 0u;
+    for (int w = threadIdx.x; w < 2 * S::NT2 * S::NP * S::DS / 4; w += S::T) z[w] = 0u;
     __syncthreads();
     for (int idx = threadIdx.x; idx < n * n; idx += S::T) {
         const int x = idx / n, y = idx - x * n;
         sm[S::oD + S::loc(x) * S::DS + S::loc(y)] = (uint8_t)D[idx];
         sm[S::oF + x * S::DS + y] = (uint8_t)F[idx];
+        if constexpr (S::ASYM) {
+            sm[S::oD + S::TT + S::loc(y) * S::DS + S::loc(x)] = (uint8_t)D[idx];
+            sm[S::oF + S::TT + y * S::DS + x] = (uint8_t)F[idx];
+        }
     }
     __syncthreads();
     if constexpr (S::REGS) {
@@ -247,10 +270,12 @@ __device__ __forceinline__ void mm_products(unsigned char *sm, int w, const uint
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc[jt][nt][e] = 0.0f;
 #pragma unroll
-    for (int s = 0; s < S::MT; ++s) {
+    for (int d = 0; d < S::NT2 * S::MT; ++d) {
+        const int s = d % S::MT, tr = d / S::MT;  // the second half: the transposes
         uint2 b[NT];
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt) b[nt] = *reinterpret_cast<const uint2 *>(v + 8 * nt * S::VS + 32 * s);
+        for (int nt = 0; nt < NT; ++nt)
+            b[nt] = *reinterpret_cast<const uint2 *>(v + tr * S::VT + 8 * nt * S::VS + 32 * s);
 #pragma unroll
         for (int jt = 0; jt < S::JT; ++jt) {
             const int m = m0 + jt * (S::NW / 2);
@@ -260,7 +285,7 @@ __device__ __forceinline__ void mm_products(unsigned char *sm, int w, const uint
                 for (int nt = 0; nt < NT; ++nt) mma_f16(acc[jt][nt], A[jt][s], b[nt]);
             } else {
                 uint32_t a[4];
-                mm_frag<S::DS>(tab, 16 * m, s, lane, a);
+                mm_frag<S::DS>(tab + tr * S::TT, 16 * m, s, lane, a);
 #pragma unroll
                 for (int nt = 0; nt < NT; ++nt) mma_f16(acc[jt][nt], a, b[nt]);
             }
@@ -284,7 +309,7 @@ __device__ __forceinline__ void mm_products(unsigned char *sm, int w, const uint
 }
 
 // p-diagonal entries of this thread's locations, h[x] = sum_y D[y][x]
-// F[p(y)][p(x)] (symmetric), from the replica's permutation bytes (integers);
+// F[p(y)][p(x)] (symmetric; general form: and the transposes'), from the replica's permutation bytes (integers);
 // one row of each table at a time.
 template <class S>
 __device__ __forceinline__ void mm_diagonal(const unsigned char *sm, const uint8_t *pb, int n, int t, int (&h)[S::K]) {
@@ -299,7 +324,10 @@ __device__ __forceinline__ void mm_diagonal(const unsigned char *sm, const uint8
     for (int y = 0; y < n; ++y) {
         const uint8_t *dr = sm + S::oD + S::loc(y) * S::DS, *fr = sm + S::oF + pb[S::pbyte(y)] * S::DS;
 #pragma unroll
-        for (int k = 0; k < K; ++k) h[k] += (int)dr[S::pos(t, k)] * (int)fr[px[k]];
+        for (int k = 0; k < K; ++k) {
+            h[k] += (int)dr[S::pos(t, k)] * (int)fr[px[k]];
+            if constexpr (S::ASYM) h[k] += (int)dr[S::TT + S::pos(t, k)] * (int)fr[S::TT + px[k]];
+        }
     }
 }
 
@@ -316,6 +344,8 @@ template <class S>
 __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int part, unsigned char *sm,
                                              const uint32_t (&A)[S::JT][S::REGS ? S::MT : 1][4]) {
     constexpr int K = S::K, LPR = S::LPR;
+    constexpr bool ASYM = S::ASYM;
+    constexpr float kScale = ASYM ? 0.5f * kMmScale : kMmScale;
     const int tid = threadIdx.x, w = __shfl_sync(kFull, tid >> 5, 0), lane = tid & 31;
     const int half = LPR == 16 ? lane >> 4 : 0;
     const int t = lane & (LPR - 1);
@@ -346,7 +376,7 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
     int32_t *gbp = a.best_perm + (size_t)r * n;
     const bool fresh = part == 0 && a.fresh;
 
-    // (|E| <= n^2 127^2 < 2^31)
+    // (|E| <= n^2 127^2 < 2^31, and twice that in the general form's sums)
     // (the best sweep and the accepted swaps stay in global memory)
     int E = 0, bestE = 0;
     bool reached = false;
@@ -396,6 +426,7 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
             sH[S::pos(t, k)] = t * K + k < n ? (float)h[k] * kMmUnit : __int_as_float(0xFF800000);
         }
         esum = mm_sum<LPR>(esum, kFull);
+        if constexpr (S::ASYM) esum >>= 1;
         if (live) {
             if (fresh) {
                 E = bestE = esum;
@@ -430,7 +461,7 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
             if (*flag) break;
         }
         // (never 0, so that an infinite energy always has weight 0)
-        const float kb = fminf(-beta_of(s) * kLog2e * kMmScale, -1e-37f);
+        const float kb = fminf(-beta_of(s) * kLog2e * kScale, -1e-37f);
         uint32_t rhi = 0;  // high words of the draws of LPR locations
         int moves = 0;
         // location i = ti K + ki
@@ -441,33 +472,43 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
             }
             const int xi = S::pos(ti, ki);
             const uint32_t aDi = base32 + S::oD + xi * S::DS;
-            const uint32_t aDr = base32 + S::oDr + par * 4 * S::NP;  // 2 D_ij units
+            const uint32_t aDr = base32 + S::oDr + par * 4 * S::NP;  // 2 D_ij (D_ij + D_ji) units
             uint2 p8 = make_uint2(0, 0);
-            int pi = 0, qb[K];
+            int pi = 0, qb[K], qt[ASYM ? K : 1];  // F_ab, F_ba of this thread's locations
             uint32_t aFi = 0;
             // ---- vectors
-            if (tid < S::NP)
-                asm volatile("st.shared.f32 [%0], %1;" ::"r"(aDr + 4 * tid), "f"((float)lds_u8(aDi + tid) * (2.0f * kMmUnit)));
+            if (tid < S::NP) {
+                const float x = ASYM ? (float)(lds_u8(aDi + tid) + lds_u8(aDi + S::TT + tid)) * kMmUnit
+                                     : (float)lds_u8(aDi + tid) * (2.0f * kMmUnit);
+                asm volatile("st.shared.f32 [%0], %1;" ::"r"(aDr + 4 * tid), "f"(x));
+            }
             if (warp_live) {
                 pi = lds_u8(aP + 8 * ti + ki);
                 p8 = lds_u64(aP + 8 * t);
                 const uint2 i8 = lds_u64(aI + 8 * t);
                 aFi = base32 + S::oF + pi * S::DS;
+                auto put = [&](uint32_t at, const int (&x)[K]) {
+#pragma unroll
+                    for (int k = 0; k + 1 < K; k += 2)
+                        asm volatile("st.shared.b32 [%0], %1;" ::"r"(at + k * 2 * LPR),
+                                     "r"(__byte_perm(x[k], x[k + 1], 0x5410)));
+                    if constexpr (K & 1)
+                        asm volatile("st.shared.b16 [%0], %1;" ::"r"(at - 2 * t + (K - 1) * 2 * LPR), "h"((uint16_t)x[K - 1]));
+                };
                 int gb[K];
 #pragma unroll
                 for (int k = 0; k < K; ++k) gb[k] = lds_u8(entry<S>(aDi, i8, k));
 #pragma unroll
                 for (int k = 0; k < K; ++k) qb[k] = lds_u8(entry<S>(aFi, p8, k));
+                put(aV + (S::oVg - S::oVq), gb);
+                put(aV, qb);
+                if constexpr (ASYM) {
 #pragma unroll
-                for (int k = 0; k + 1 < K; k += 2) {
-                    const uint32_t g2 = __byte_perm(gb[k], gb[k + 1], 0x5410), q2 = __byte_perm(qb[k], qb[k + 1], 0x5410);
-                    asm volatile("st.shared.b32 [%0], %1;" ::"r"(aV + (S::oVg - S::oVq) + k * 2 * LPR), "r"(g2));
-                    asm volatile("st.shared.b32 [%0], %1;" ::"r"(aV + k * 2 * LPR), "r"(q2));
-                }
-                if constexpr (K & 1) {
-                    asm volatile("st.shared.b16 [%0], %1;" ::"r"(aV - 2 * t + (S::oVg - S::oVq) + (K - 1) * 2 * LPR),
-                                 "h"((uint16_t)gb[K - 1]));
-                    asm volatile("st.shared.b16 [%0], %1;" ::"r"(aV - 2 * t + (K - 1) * 2 * LPR), "h"((uint16_t)qb[K - 1]));
+                    for (int k = 0; k < K; ++k) gb[k] = lds_u8(entry<S>(aDi, i8, k) + S::TT);
+#pragma unroll
+                    for (int k = 0; k < K; ++k) qt[k] = lds_u8(entry<S>(aFi, p8, k) + S::TT);
+                    put(aV + (S::oVg - S::oVq) + S::VT, gb);
+                    put(aV + S::VT, qt);
                 }
             }
             __syncthreads();
@@ -484,7 +525,8 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
                 MmVals<K> e;
                 float hk[K], mq[K];
 #pragma unroll
-                for (int k = 0; k < K; ++k) mq[k] = __int_as_float(0x4B000000 | qb[k]);  // 2^23 + F_ab
+                for (int k = 0; k < K; ++k)  // 2^23 + F_ab (F_ab + F_ba)
+                    mq[k] = __int_as_float(0x4B000000 | (ASYM ? qb[k] + qt[ASYM ? k : 0] : qb[k]));
 #pragma unroll
                 for (int k = 0; k + 1 < K; k += 2) {
                     const uint32_t x = 4 * k * LPR + 8 * t;
@@ -545,7 +587,7 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
                 int v = __shfl_sync(kFull, (t << 8) | kk | (int)(__byte_perm(p8.x, p8.y, kk) << 16), __ffs(ball) - 1);
                 if (__any_sync(kFull, ball == 0)) {
                     const uint32_t dlo = philox4x32_10(a.inst, grep, (uint32_t)s, (uint32_t)i, a.key0, a.key1).x;
-                    const int js = mm_exact_draw<K, LPR>(e, n, t, beta_of(s), ((unsigned long long)dhi << 32) | dlo, kFull);
+                    const int js = mm_exact_draw<K, LPR>(e, n, t, kScale, beta_of(s), ((unsigned long long)dhi << 32) | dlo, kFull);
                     if (ball == 0) {
                         const int tx = js / K, kx = js - tx * K;
                         v = (tx << 8) | kx | (lds_u8(aP + 8 * tx + kx) << 16);
@@ -559,34 +601,63 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
                     const int xj = S::pos(tj, kj);
                     const uint32_t aFj = base32 + S::oF + fb * S::DS, aDj = base32 + S::oD + xj * S::DS;
                     const float rs = lds_f32(aR + 4 * fb), cs = lds_f32(aC + 4 * xj), hs = lds_f32(aH + 4 * xj);
-                    const float dq = 0.5f * lds_f32(aDr + 4 * xj) * (float)lds_u8(aFi + fb);  // D_ij F_ab
+                    // what the swap adds to both moved entries of h: D_ij F_ab (D_ij F_ba + D_ji F_ab)
+                    float dq, dd;
+                    if constexpr (ASYM) {
+                        const int fab = lds_u8(aFi + fb), fba = lds_u8(aFi + S::TT + fb);
+                        dq = (float)(lds_u8(aDi + xj) * fba + lds_u8(aDi + S::TT + xj) * fab) * kMmUnit;
+                        dd = lds_f32(aDr + 4 * xj) * (float)(fab + fba);
+                    } else {
+                        dq = 0.5f * lds_f32(aDr + 4 * xj) * (float)lds_u8(aFi + fb);
+                        dd = 2.0f * dq;
+                    }
                     // h[m] += (D_im - D_jm) (F_b,p(m) - F_a,p(m))
                     float2 hn[K / 2 + 1];
+                    auto word = [&](uint32_t at) {  // a pair of a row of D at this thread's locations
+                        uint32_t x;
+                        asm volatile("ld.shared.u16 %0, [%1];" : "=r"(x) : "r"(at + 2 * t));
+                        return x;
+                    };
+                    auto units = [](uint32_t x) {  // 2^-25 + entry units
+                        return make_float2(__int_as_float((int)__byte_perm(x, 0x33000000u, 0x7540)),
+                                           __int_as_float((int)__byte_perm(x, 0x33000000u, 0x7541)));
+                    };
+                    auto ones = [](int x) { return __int_as_float(0x4B000000 | x); };  // 2^23 + entry
 #pragma unroll
                     for (int k = 0; k + 1 < K; k += 2) {
-                        uint32_t dj;
-                        asm volatile("ld.shared.u16 %0, [%1];" : "=r"(dj) : "r"(aDj + k * LPR + 2 * t));
-                        // 2^-25 + D_jm units
-                        const float2 mj = make_float2(__int_as_float((int)__byte_perm(dj, 0x33000000u, 0x7540)),
-                                                      __int_as_float((int)__byte_perm(dj, 0x33000000u, 0x7541)));
-                        const float2 u = sub2(fma2(lds_f64(aDr + 4 * k * LPR + 8 * t), two(0.5f), two(kMmOne)), mj);
-                        const float2 vv = sub2(make_float2(__int_as_float(0x4B000000 | lds_u8(entry<S>(aFj, p8, k))),
-                                                           __int_as_float(0x4B000000 | lds_u8(entry<S>(aFj, p8, k + 1)))),
-                                               make_float2(mq[k], mq[k + 1]));
-                        hn[k / 2] = fma2(u, vv, make_float2(hk[k], hk[k + 1]));
+                        float2 u;
+                        if constexpr (ASYM)
+                            u = sub2(units(word(aDi + k * LPR)), units(word(aDj + k * LPR)));
+                        else
+                            u = sub2(fma2(lds_f64(aDr + 4 * k * LPR + 8 * t), two(0.5f), two(kMmOne)),
+                                     units(word(aDj + k * LPR)));
+                        const float2 fbk = make_float2(ones(lds_u8(entry<S>(aFj, p8, k))), ones(lds_u8(entry<S>(aFj, p8, k + 1))));
+                        const float2 fak = ASYM ? make_float2(ones(qb[k]), ones(qb[k + 1])) : make_float2(mq[k], mq[k + 1]);
+                        float2 x = fma2(u, sub2(fbk, fak), make_float2(hk[k], hk[k + 1]));
+                        if constexpr (ASYM) {
+                            const float2 ut = sub2(units(word(aDi + S::TT + k * LPR)), units(word(aDj + S::TT + k * LPR)));
+                            const float2 ft = make_float2(ones(lds_u8(entry<S>(aFj, p8, k) + S::TT)),
+                                                          ones(lds_u8(entry<S>(aFj, p8, k + 1) + S::TT)));
+                            x = fma2(ut, sub2(ft, make_float2(ones(qt[k]), ones(qt[k + 1]))), x);
+                        }
+                        hn[k / 2] = x;
                     }
                     if constexpr (K & 1) {
                         constexpr int k = K - 1;
-                        const float mj = __int_as_float(0x33000000 | lds_u8(aDj + k * LPR + t));
-                        const float vv = __int_as_float(0x4B000000 | lds_u8(entry<S>(aFj, p8, k))) - mq[k];
-                        hn[K / 2].x = fmaf(fmaf(lds_f32(aDr + 4 * (k * LPR + t)), 0.5f, kMmOne) - mj, vv, hk[k]);
+                        auto unit = [&](uint32_t row) { return __int_as_float(0x33000000 | lds_u8(row + k * LPR + t)); };
+                        const float u = (ASYM ? unit(aDi) : fmaf(lds_f32(aDr + 4 * (k * LPR + t)), 0.5f, kMmOne)) - unit(aDj);
+                        float x = fmaf(u, ones(lds_u8(entry<S>(aFj, p8, k))) - (ASYM ? ones(qb[k]) : mq[k]), hk[k]);
+                        if constexpr (ASYM)
+                            x = fmaf(unit(aDi + S::TT) - unit(aDj + S::TT),
+                                     ones(lds_u8(entry<S>(aFj, p8, k) + S::TT)) - ones(qt[k]), x);
+                        hn[K / 2].x = x;
                     }
                     __syncwarp();  // reads of h and p by the replica's threads done
                     if (sw) {
 #pragma unroll
                         for (int k = 0; k + 1 < K; k += 2) *reinterpret_cast<float2 *>(sH + k * LPR + 2 * t) = hn[k / 2];
                         if constexpr (K & 1) sH[(K - 1) * LPR + t] = hn[K / 2].x;
-                        E += (int)(((rs - hi) + (cs - hs) + 2.0f * dq) * kMmScale);
+                        E += (int)(((rs - hi) + (cs - hs) + dd) * kScale);
                         moves += 1;
                     }
                     __syncwarp();
@@ -632,6 +703,7 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
 #pragma unroll
             for (int k = 0; k < K; ++k) eq1 += h[k];
             eq1 = mm_sum<LPR>(eq1, kFull);
+            if constexpr (S::ASYM) eq1 >>= 1;
             if (live && t == 0 && eq1 != E) atomicOr(a.status, 1);
         }
         if (live) {
@@ -720,9 +792,9 @@ struct MmCall {
     int *batch_blocks = nullptr;
 };
 
-template <int K, int LPR>
+template <int K, int LPR, bool ASYM>
 static int mm_one(const MmCall &c) {
-    using S = MmShape<K, LPR>;
+    using S = MmShape<K, LPR, ASYM>;
     const bool batch = c.descs || c.batch_blocks;
     const cudaError_t e =
         batch ? cudaFuncSetAttribute(mm_batch_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::bytes)
@@ -745,47 +817,55 @@ static int mm_one(const MmCall &c) {
     return (int)cudaGetLastError();
 }
 
-static int mm_dispatch(int n, const MmCall &c) {
-    if (n <= 32 || n > 256) return (int)cudaErrorInvalidValue;
+template <bool ASYM>
+static int mm_dispatch_form(int n, const MmCall &c) {
     if (n <= 128) {
         switch ((n + 15) / 16) {
-        case 3: return mm_one<3, 16>(c);
-        case 4: return mm_one<4, 16>(c);
-        case 5: return mm_one<5, 16>(c);
-        case 6: return mm_one<6, 16>(c);
-        case 7: return mm_one<7, 16>(c);
-        default: return mm_one<8, 16>(c);
+        case 3: return mm_one<3, 16, ASYM>(c);
+        case 4: return mm_one<4, 16, ASYM>(c);
+        case 5: return mm_one<5, 16, ASYM>(c);
+        case 6: return mm_one<6, 16, ASYM>(c);
+        case 7: return mm_one<7, 16, ASYM>(c);
+        default: return mm_one<8, 16, ASYM>(c);
         }
     }
-    switch ((n + 31) / 32) {
-    case 5: return mm_one<5, 32>(c);
-    case 6: return mm_one<6, 32>(c);
-    case 7: return mm_one<7, 32>(c);
-    default: return mm_one<8, 32>(c);
+    if ((n + 31) / 32 == 5) return mm_one<5, 32, ASYM>(c);
+    if constexpr (!ASYM) {  // (the general form's four tables end at 160 locations)
+        switch ((n + 31) / 32) {
+        case 6: return mm_one<6, 32, ASYM>(c);
+        case 7: return mm_one<7, 32, ASYM>(c);
+        default: return mm_one<8, 32, ASYM>(c);
+        }
     }
+    return (int)cudaErrorInvalidValue;
 }
 
-int mm_query(int n, MmInfo *info) {
+static int mm_dispatch(int n, bool asym, const MmCall &c) {
+    if (n <= 32 || n > (asym ? kMmGeneralMax : 256)) return (int)cudaErrorInvalidValue;
+    return asym ? mm_dispatch_form<true>(n, c) : mm_dispatch_form<false>(n, c);
+}
+
+int mm_query(int n, bool asym, MmInfo *info) {
     MmCall c;
     c.info = info;
-    return mm_dispatch(n, c);
+    return mm_dispatch(n, asym, c);
 }
 
-int mm_launch(const SweepArgs &a, int grid, cudaStream_t st) {
+int mm_launch(const SweepArgs &a, bool asym, int grid, cudaStream_t st) {
     MmCall c;
     c.args = &a;
     c.grid = grid;
     c.st = st;
-    return mm_dispatch(a.n, c);
+    return mm_dispatch(a.n, asym, c);
 }
 
-int mm_batch_blocks_per_sm(int n, int *blocks) {
+int mm_batch_blocks_per_sm(int n, bool asym, int *blocks) {
     MmCall c;
     c.batch_blocks = blocks;
-    return mm_dispatch(n, c);
+    return mm_dispatch(n, asym, c);
 }
 
-int mm_batch_launch(int n, const SweepArgs *descs, const BatchUnit *units, int nunits, int *queue, int grid,
+int mm_batch_launch(int n, bool asym, const SweepArgs *descs, const BatchUnit *units, int nunits, int *queue, int grid,
                     cudaStream_t st) {
     MmCall c;
     c.descs = descs;
@@ -794,7 +874,7 @@ int mm_batch_launch(int n, const SweepArgs *descs, const BatchUnit *units, int n
     c.queue = queue;
     c.grid = grid;
     c.st = st;
-    return mm_dispatch(n, c);
+    return mm_dispatch(n, asym, c);
 }
 
 }  // namespace pdit

@@ -1744,17 +1744,19 @@ struct SmallInfo {
 int small_query(int n, bool f32, int warps, SmallInfo *info);
 int small_launch(const SweepArgs &a, bool f32, int grid, int warps, cudaStream_t stream);
 
-// Tensor-core product kernel (pdit_mma.cu): symmetric instances with zero
-// diagonals and entries in 0..127; one compiled kernel per range of n.
+// Tensor-core product kernel (pdit_mma.cu): zero diagonals and entries in
+// 0..127, symmetric or (up to kMmGeneralMax locations) general; one compiled
+// kernel per range of n.
 // Return a cudaError_t value.
 struct MmInfo {
     int threads, slots, lanes, k, blocks_per_sm;  // slots: replicas per CTA; lanes: threads per replica
     size_t smem;
 };
-int mm_query(int n, MmInfo *info);
-int mm_launch(const SweepArgs &a, int grid, cudaStream_t stream);
-int mm_batch_blocks_per_sm(int n, int *blocks);
-int mm_batch_launch(int n, const SweepArgs *descs, const BatchUnit *units, int nunits, int *queue, int grid,
+constexpr int kMmGeneralMax = 160;
+int mm_query(int n, bool asym, MmInfo *info);
+int mm_launch(const SweepArgs &a, bool asym, int grid, cudaStream_t stream);
+int mm_batch_blocks_per_sm(int n, bool asym, int *blocks);
+int mm_batch_launch(int n, bool asym, const SweepArgs *descs, const BatchUnit *units, int nunits, int *queue, int grid,
                     cudaStream_t stream);
 
 }  // namespace pdit

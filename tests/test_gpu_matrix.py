@@ -1,5 +1,5 @@
-"""GPU parity of the tensor-core product kernel (symmetric instances with zero
-diagonals and entries in 0..127, above the sizes of the one-warp kernels):
+"""GPU parity of the tensor-core product kernel (instances with zero diagonals
+and entries in 0..127, symmetric or general, above the sizes of the small kernel):
 sizes at the edges of its compiled ranges, blocks with one replica, with a
 part of their slots and with all of them, entries at the ends of their range,
 and where the automatic choice takes it. Every replica compared equals the
@@ -88,3 +88,24 @@ def test_entry_range(hi):
                  np.full(S, 1e30, np.float32)):
         g, _ = run(D, F, beta, S, 4, 6)
         check(g, D, F, beta, S, 4, 0, 6)
+
+
+@pytest.mark.parametrize("n", [33, 48, 49, 64, 65, 80, 81, 96, 97, 112, 113, 128, 129, 160])
+def test_general_form_size_edges(n):
+    D, F = G.asymmetric(n, 0, 99, n, 101), G.asymmetric(n, 0, 99, n, 103)
+    S = 5
+    beta = O.beta_schedule("linear", S, O.beta_max(D, F))
+    g, _ = run(D, F, beta, S, 3, 5)
+    check(g, D, F, beta, S, 3, 0, 5)
+
+
+@pytest.mark.parametrize("n,per_sm", [(50, 9), (100, 27), (120, 3), (150, 12)])
+def test_general_form_block_fill(n, per_sm):
+    D, F = G.asymmetric_instance(n, seed=n)
+    S = 3
+    beta = O.beta_schedule("geometric", S, O.beta_max(D, F))
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    R = sms * per_sm - per_sm // 2
+    g, _ = run(D, F, beta, S, 8, R)
+    for lo, hi in ((0, min(R, 32)), (R // 2, R // 2 + 4), (R - 6, R)):
+        check(g, D, F, beta, S, 8, lo, hi)
