@@ -661,13 +661,11 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
                         moves += 1;
                     }
                     __syncwarp();
-                    if (sw && t == 0) {
-                        sH[xi] = rs + dq;
-                        sH[xj] = cs + dq;
-                        pb[8 * ti + ki] = (uint8_t)fb;
-                        pb[8 * tj + kj] = (uint8_t)pi;
-                        ib[S::ibyte(pi)] = (uint8_t)xj;
-                        ib[S::ibyte(fb)] = (uint8_t)xi;
+                    if (sw && t < 2) {  // one moved facility and location each
+                        const bool first = t == 0;
+                        sH[first ? xi : xj] = (first ? rs : cs) + dq;
+                        pb[first ? 8 * ti + ki : 8 * tj + kj] = (uint8_t)(first ? fb : pi);
+                        ib[S::ibyte(first ? fb : pi)] = (uint8_t)(first ? xi : xj);
                     }
                     __syncwarp();
                     if (live && E < bestE) {

@@ -285,7 +285,7 @@ __device__ __forceinline__ void fisher_yates(const SweepArgs &a, uint32_t grep, 
 // eq5_draw_exact computes just that. eq5_draw_core first draws with binary32
 // weights w_j = 2^(-beta log2(e) dc_j) (the stay outcome, dc = 0, is the
 // reference: no minimum is needed), their prefix sums and t = u total, and
-// keeps the outcome only if t - m and t + m, m = 2^-15 total, both fall
+// keeps the outcome only if t - m and t + m, m = 2^-16 total, both fall
 // inside its interval; otherwise (and when total >= 2^64, infinite or not a
 // number) the exact draw decides. Both prefix distributions approximate that
 // of e^(-beta dc_j):
@@ -293,16 +293,17 @@ __device__ __forceinline__ void fisher_yates(const SweepArgs &a, uint32_t grep, 
 //     its reduction, < 2^-20, the weights cut beyond 40 and the truncation,
 //     < 2^-40: relative 6e-6 a weight;
 //   binary32: arguments that matter lie in [-40, 64] (total < 2^64; terms
-//     below 2^-40 of the stay weight carry nothing) and have four roundings,
-//     64 x 3.5 x 2^-24 x ln 2 = 9.3e-6, and ex2.approx, 2^-22: 9.6e-6.
+//     below 2^-40 of the stay weight carry nothing) and have three roundings
+//     and a rounded log2(e), 64 x 3.25 x 2^-24 x ln 2 = 8.6e-6, and
+//     ex2.approx, 2^-22: 8.8e-6.
 // A prefix share F = A/(A+B) moves by F (1 - F) times the difference of the
-// relative errors, at most half of each bound, 7.8e-6 together; the binary32
-// sums add at most 20 roundings, 1.2e-6, twice, and u and t 2 x 2^-24. The
-// sum, 1.1e-5, is a third of 2^-15, so a kept outcome is the exact one. The
-// exact draw runs where t lies within m of a boundary: at most 2^-14 per
-// boundary that carries weight (0.6% of draws at n = 100 and beta = 0).
+// relative errors, at most half of each bound, 7.4e-6 together; the binary32
+// sums add at most 14 roundings, 8.4e-7, twice, and u and t 2 x 2^-24. The
+// sum, 9.2e-6, is below 2^-16 = 1.53e-5, so a kept outcome is the exact one.
+// The exact draw runs where t lies within m of a boundary: at most 2^-15 per
+// boundary that carries weight (0.3% of draws at n = 100 and beta = 0).
 // ---------------------------------------------------------------------------
-constexpr float kDrawMargin = 3.0517578125e-05f;   // 2^-15
+constexpr float kDrawMargin = 1.52587890625e-05f;   // 2^-16
 constexpr float kDrawLimit = 1.8446744073709552e19f;  // 2^64
 constexpr float kLog2e = 1.44269502f;
 
