@@ -99,6 +99,7 @@ struct Plan {
     bool mm = false;  // with dot: the tensor-core product kernel (pdit_mma.cu)
     int lanes = 32;   // its threads per replica
     bool small = false;  // the small kernel (pdit_small.cu)
+    bool cc = false;     // the concurrent-update kernel (pdit_concurrent.cu)
     int stride = 0, sv_len = 0, cupim_off = 0, v2_off = 0, rc_off = 0, dstride = 0;
     size_t table_elems = 0;  // int32 entries of one replica's saved table (workspace)
     size_t df_bytes = 0, group_bytes = 0, smem = 0;
@@ -455,6 +456,32 @@ bool use_small_path(const pdit_qap *h, const pdit_opts *o) {
            h->force_pk <= 1 && h->force_place != PDIT_PLACE_GLOBAL && h->force_infl != PDIT_INFLUENCE_PRODUCTS;
 }
 
+// Launch shape of the concurrent-update kernel: one CTA per replica.
+int make_cc_plan(const pdit_qap *h, int replicas, Plan *p) {
+    pdit::CcInfo info{};
+    const int e = pdit::concurrent_query(h->n, &info);
+    if (e != 0) return cuda_fail((cudaError_t)e, "occupancy query");
+    if (info.blocks_per_sm < 1 || info.smem > h->smem_optin) return PDIT_ENOTSUP;
+    p->cc = true;
+    p->tsmem = true;
+    p->pk = p->wpr = p->maxk = 1;
+    p->table_elems = 0;
+    p->groups = 1;
+    p->threads = info.threads;
+    p->smem = info.smem;
+    p->grid = std::max(1, std::min(replicas, h->num_sms * info.blocks_per_sm));
+    return PDIT_OK;
+}
+
+// Whether a call runs the concurrent-update kernel: mode 3 of a symmetric
+// instance with zero diagonals and entries in 0..127, no table dump, and no
+// setting that shapes the table kernels.
+bool use_cc_path(const pdit_qap *h, const pdit_opts *o) {
+    return o->mode == PDIT_MODE_CUPIM && h->n <= pdit::kCcMax && !h->asym && h->zero_diag && h->dt_bytes == 1 &&
+           h->nonneg && !o->tables && h->force_wpr == 0 && h->force_pk == 0 && h->force_groups == 0 &&
+           h->force_place == PDIT_PLACE_AUTO && h->force_infl == PDIT_INFLUENCE_AUTO;
+}
+
 // The product kernel of a call: tensor-core products where the instance
 // allows them and no wider mapping than a warp per replica is asked for, else
 // the dot-product kernel. `any`: also where the automatic rule prefers the
@@ -482,6 +509,11 @@ bool use_dot_path(const pdit_qap *h, const pdit_opts *o) {
 // the table kernels.
 int plan_for(const pdit_qap *h, const pdit_opts *o, Plan *p) {
     if (use_class_path(h, o)) return make_class_plan(h, o->replicas, h->force_wpr, p);
+    if (use_cc_path(h, o)) {
+        const int rc = make_cc_plan(h, o->replicas, p);
+        if (rc != PDIT_ENOTSUP) return rc;
+        *p = Plan();
+    }
     if (use_small_path(h, o)) {
         const int rc = make_small_plan(h, o->replicas, p);
         if (rc != PDIT_ENOTSUP) return rc;
@@ -564,7 +596,7 @@ int parts_of(const pdit_opts *o, const Plan &p, int span) {
 // kept between calls by the server, the dot kernel's permuted flow matrix;
 // either kernel's table between the parts of a launch).
 bool needs_tables(const pdit_opts *o, const Plan &p, bool persist = false, bool whole = false) {
-    if (p.mm || p.small) return false;  // their state is the permutation and the energies
+    if (p.mm || p.small || p.cc) return false;  // their state is the permutation and the energies
     return persist || o->mode == PDIT_MODE_PT || (!p.dot && !p.tsmem) || (!whole && may_split(o, p));
 }
 
@@ -1086,6 +1118,7 @@ int pdit_anneal_ex(pdit_qap *h, const pdit_opts *o) {
             PDIT_CK(cudaMemsetAsync(w.queue, 0, sizeof(int32_t), st));
             if (a.segments > 1) PDIT_CK(cudaMemsetAsync(w.seg_done, 0, sizeof(int32_t) * R, st));
             const int e = plan.cls ? class_launch(h->dt_bytes, plan, a, st)
+                        : plan.cc ? pdit::concurrent_launch(a, plan.grid, st)
                         : plan.small ? pdit::small_launch(a, h->f32_ok != 0, plan.grid, plan.groups, st)
                         : plan.mm  ? pdit::mm_launch(a, h->asym != 0, plan.grid, st)
                         : plan.dot ? pdit::dot_launch(plan.maxk, plan.wpr, a, plan.grid, plan.threads, plan.smem, st)

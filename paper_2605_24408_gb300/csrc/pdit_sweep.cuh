@@ -1760,4 +1760,15 @@ int mm_batch_blocks_per_sm(int n, bool asym, int *blocks);
 int mm_batch_launch(int n, bool asym, const SweepArgs *descs, const BatchUnit *units, int nunits, int *queue, int grid,
                     cudaStream_t stream);
 
+// Concurrent-update kernel (pdit_concurrent.cu): mode 3 of symmetric instances
+// with zero diagonals and entries in 0..127, one CTA per replica. Return a
+// cudaError_t value.
+struct CcInfo {
+    int threads, blocks_per_sm;
+    size_t smem;
+};
+constexpr int kCcMax = 128;  // locations
+int concurrent_query(int n, CcInfo *info);
+int concurrent_launch(const SweepArgs &a, int grid, cudaStream_t stream);
+
 }  // namespace pdit
