@@ -25,8 +25,12 @@
 // that is the set the greedy pass in priority order accepts. Acceptance and
 // energies are exact, so the trajectories equal the table kernels'.
 //
-// N = 100, 4096 replicas x 100 iterations: 13.3 ms (33.7 ms with the table
-// kernels, which update every table entry for every accepted swap).
+// Bound: an iteration's latency, about 17000 clocks at N = 100, 7000 of them
+// the product (two warps a scheduler reach half of mma.sync's rate; loads of a
+// step ahead of its products made no difference) and 2000 to 4000 the
+// matching, two CTAs an SM overlapped. N = 100, 4096 replicas x 60 iterations:
+// 7.8 ms (21.6 ms with the table kernels, which update every table entry for
+// every accepted swap); N = 12, 64 replicas: 0.21 ms (0.57 ms).
 #include "pdit_f16.cuh"
 #include "pdit_sweep.cuh"
 
@@ -37,6 +41,7 @@ struct CcShape {
     static constexpr int MT = MT_, NT = 2 * MT, NP = 16 * MT, T = 32 * MT, LC = 4 * MT;
     static constexpr int GS = 16 * (MT | 1);  // row stride of D and G, bytes
     static constexpr int FS = 256;            // of F: an entry's address is its row's with the column for the low byte
+    static constexpr int CTAS = (MT >= 7 ? 512 : MT >= 5 ? 640 : 768) / T;  // resident CTAs an SM aimed at (more spill)
     // shared memory, bytes (F first: its rows are 256-byte aligned)
     static constexpr int oF = 0, oD = oF + NP * FS, oG = oD + NP * GS, oP = oG + NP * GS, oS = oP + 128,
                          oB = oS + 4 * (NP + 8), oTk = oB + 2 * 4 * 128, oX = oTk + 128, bytes = oX + 32;
@@ -256,14 +261,15 @@ __device__ __forceinline__ void cc_run_replica(const SweepArgs &a, int r, int pa
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int i = row0 + 2 * h;
-            float pre[LC], lsum = 0.0f;
+            // prefix sums of four outcomes each (the draw's at most 17
+            // roundings, 1.0e-6 of the total, leave 1.5e-5 its slack)
+            float pre[S::MT], lsum = 0.0f;
 #pragma unroll
-            for (int k = 0; k < NT; ++k) {
-                const float2 x = make_float2(e[k][2 * h] * kb, e[k][2 * h + 1] * kb);
-                lsum += ex2_approx(x.x);
-                pre[2 * k] = lsum;
-                lsum += ex2_approx(x.y);
-                pre[2 * k + 1] = lsum;
+            for (int k = 0; k < S::MT; ++k) {
+                const float2 x = mul2(make_float2(e[2 * k][2 * h], e[2 * k][2 * h + 1]), two(kb));
+                const float2 y = mul2(make_float2(e[2 * k + 1][2 * h], e[2 * k + 1][2 * h + 1]), two(kb));
+                lsum += (ex2_approx(x.x) + ex2_approx(x.y)) + (ex2_approx(y.x) + ex2_approx(y.y));
+                pre[k] = lsum;
             }
             float incl = lsum;
 #pragma unroll
@@ -276,19 +282,35 @@ __device__ __forceinline__ void cc_run_replica(const SweepArgs &a, int r, int pa
             const float tt = __uint2float_rn(dhi >> 8) * 5.9604644775390625e-08f * total;
             const float mg = total < kDrawLimit ? kDrawMargin * total : __int_as_float(0x7FC00000);
             const float base = (incl - lsum) - tt;
-            float near = fabsf(base), z = base, dsel = 0.0f;
+            // the four outcomes around the draw, then the one: boundaries lo < 0 < hi
+            float lo = base, v[4] = {e[0][2 * h], e[0][2 * h + 1], e[1][2 * h], e[1][2 * h + 1]};
             int kk = 0;
 #pragma unroll
-            for (int k = 0; k < LC; ++k) {
+            for (int k = 1; k < S::MT; ++k) {
+                const float z = pre[k - 1] + base;
                 if (z < 0.0f) {
-                    kk = k;
-                    dsel = e[k / 2][2 * h + (k & 1)];
+                    lo = z;
+                    kk = 4 * k;
+                    v[0] = e[2 * k][2 * h];
+                    v[1] = e[2 * k][2 * h + 1];
+                    v[2] = e[2 * k + 1][2 * h];
+                    v[3] = e[2 * k + 1][2 * h + 1];
                 }
-                z = pre[k] + base;
-                near = fminf(near, fabsf(z));
+            }
+            float hi = lo + ex2_approx(v[0] * kb), dsel = v[0];
+            const int k4 = kk;
+#pragma unroll
+            for (int k = 1; k < 4; ++k) {
+                const float z = hi + ex2_approx(v[k] * kb);
+                if (hi < 0.0f) {
+                    lo = hi;
+                    hi = z;
+                    kk = k4 + k;
+                    dsel = v[k];
+                }
             }
             // the lane whose interval certainly holds the draw (eq5_draw_core)
-            const unsigned ball = __ballot_sync(kFull, base < 0.0f && z > 0.0f && near > mg);
+            const unsigned ball = __ballot_sync(kFull, fminf(-lo, hi) > mg);
             const unsigned mine = (ball >> (lane & 28)) & 15u;
             int src = __ffs(mine) - 1;
             int js = __shfl_sync(kFull, LC * q + kk, src, 4);
@@ -384,7 +406,7 @@ __device__ __forceinline__ void cc_run_replica(const SweepArgs &a, int r, int pa
 // replica before part k + 1; see dot_kernel for why the wait for the part
 // before ends.
 template <class S>
-__global__ void __launch_bounds__(S::T, 512 / S::T) concurrent_kernel(const SweepArgs a) {
+__global__ void __launch_bounds__(S::T, S::CTAS) concurrent_kernel(const SweepArgs a) {
     extern __shared__ __align__(1024) unsigned char smem[];
     for (int w = threadIdx.x; w < S::oP / 4; w += S::T) reinterpret_cast<uint32_t *>(smem)[w] = 0u;
     __syncthreads();
