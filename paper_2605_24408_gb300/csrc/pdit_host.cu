@@ -30,6 +30,7 @@ struct pdit_qap {
     uint8_t *dx = nullptr;  // x_c on the device
     int f32_ok = 0;         // 8 (n + 2) max|D| max|F| < 2^24: every entry and energy exact in binary32
     int nonneg = 0;         // every entry of D and F >= 0
+    int64_t top = 0;        // the largest |entry| of D and F
     int packed_ok = 0;      // max-min of D and of F <= 127: swap factors fit int8
     std::vector<int32_t> hD, hF;
     std::vector<uint8_t> cls_x;  // class bit of every facility (two-level flows)
@@ -98,6 +99,7 @@ struct Plan {
     bool tsmem = true, cls = false, dot = false;
     bool mm = false;  // with dot: the tensor-core product kernel (pdit_mma.cu)
     int lanes = 32;   // its threads per replica
+    int form = 0;     // its form
     bool small = false;  // the small kernel (pdit_small.cu)
     bool cc = false;     // the concurrent-update kernel (pdit_concurrent.cu)
     int stride = 0, sv_len = 0, cupim_off = 0, v2_off = 0, rc_off = 0, dstride = 0;
@@ -369,12 +371,19 @@ int make_dot_plan(const pdit_qap *h, int replicas, int wpr, Plan *p, size_t rese
     return PDIT_OK;
 }
 
-// Whether an instance can run the tensor-core product kernel: zero diagonals
-// and every entry of D and F in 0..127; the general form also with every
-// energy below 2^24 and up to the sizes whose four tables fit.
+// The product kernel's form of an instance (pdit_mma.cu).
+int mm_form(const pdit_qap *h) {
+    return h->asym ? pdit::kMmGeneral : h->dt_bytes == 1 ? pdit::kMmSymmetric : pdit::kMmWide;
+}
+
+// Whether an instance can run the tensor-core product kernel: zero diagonals,
+// a size with a compiled kernel and every entry of D and F in 0..127; the
+// general form also with every energy below 2^24, the symmetric one with
+// entries to 2047 too.
 bool mm_eligible(const pdit_qap *h) {
-    if (!h->zero_diag || h->dt_bytes != 1 || !h->nonneg || h->n <= 32) return false;
-    return !h->asym || (h->f32_ok && h->n <= pdit::kMmGeneralMax);
+    if (!h->zero_diag || !h->nonneg || h->n <= 32 || h->n > pdit::kMmMax[mm_form(h)]) return false;
+    if (h->asym) return h->dt_bytes == 1 && h->f32_ok;
+    return h->dt_bytes == 1 || h->top <= pdit::kMmWideTop;
 }
 
 // Launch shape of the tensor-core product kernel: its thread mapping and
@@ -382,7 +391,7 @@ bool mm_eligible(const pdit_qap *h) {
 // over the GPU.
 int make_mm_plan(const pdit_qap *h, int replicas, Plan *p, size_t reserve = 0) {
     pdit::MmInfo info{};
-    const int e = pdit::mm_query(h->n, h->asym != 0, &info);
+    const int e = pdit::mm_query(h->n, mm_form(h), &info);
     if (e != 0) return cuda_fail((cudaError_t)e, "occupancy query");
     if (info.blocks_per_sm < 1 || info.smem + reserve > h->smem_optin) return PDIT_ENOTSUP;
     p->dot = p->mm = true;
@@ -391,6 +400,7 @@ int make_mm_plan(const pdit_qap *h, int replicas, Plan *p, size_t reserve = 0) {
     p->wpr = 1;
     p->maxk = info.k;
     p->lanes = info.lanes;
+    p->form = mm_form(h);
     p->table_elems = 0;
     p->threads = info.threads;
     p->smem = info.smem;
@@ -492,7 +502,7 @@ int product_plan(const pdit_qap *h, int replicas, Plan *p, size_t reserve, bool 
         if (rc != PDIT_ENOTSUP) return rc;
         *p = Plan();
     }
-    if (h->asym) return PDIT_ENOTSUP;
+    if (!dot_eligible(h)) return PDIT_ENOTSUP;
     return any ? make_dot_plan(h, replicas, h->force_wpr, p, reserve) : auto_dot_plan(h, replicas, p, reserve);
 }
 
@@ -892,6 +902,7 @@ int qap_prepare(int n, const int32_t *D, const int32_t *F, pdit_qap **out) {
     h->nonneg = dlo >= 0 && flo >= 0 ? 1 : 0;
     h->packed_ok = (dhi - dlo <= 127 && fhi - flo <= 127) ? 1 : 0;
     const int64_t mx = std::max(maxd, maxf);
+    h->top = mx;
     h->dt_bytes = mx <= 127 ? 1 : (mx <= 32767 ? 2 : 4);
     h->hD.assign(D, D + (size_t)n * n);
     h->hF.assign(F, F + (size_t)n * n);
@@ -1120,7 +1131,7 @@ int pdit_anneal_ex(pdit_qap *h, const pdit_opts *o) {
             const int e = plan.cls ? class_launch(h->dt_bytes, plan, a, st)
                         : plan.cc ? pdit::concurrent_launch(a, plan.grid, st)
                         : plan.small ? pdit::small_launch(a, h->f32_ok != 0, plan.grid, plan.groups, st)
-                        : plan.mm  ? pdit::mm_launch(a, h->asym != 0, plan.grid, st)
+                        : plan.mm  ? pdit::mm_launch(a, mm_form(h), plan.grid, st)
                         : plan.dot ? pdit::dot_launch(plan.maxk, plan.wpr, a, plan.grid, plan.threads, plan.smem, st)
                                    : sweep_launch(h->dt_bytes, h->asym != 0, plan, a, st);
             if (e != 0) return cuda_fail((cudaError_t)e, "sweep kernel launch");
@@ -1567,7 +1578,7 @@ struct BatchOut {
 struct BatchClass {
     int dt = 1, maxk = 1, wpr = 1, pk = 1;
     bool tsmem = true, asym = false, dot = false, mm = false;
-    int lanes = 32, n = 0;  // mm: threads per replica, the size of one of its instances
+    int lanes = 32, form = 0, n = 0;  // mm: threads per replica, form, the size of one of its instances
     int threads = 32, grid = 1, nunits = 0;
     size_t smem = 0;
     std::vector<int> items;
@@ -1584,7 +1595,7 @@ int batch_blocks_t(const BatchClass &c, int *blocks) {
 }
 
 int batch_blocks(const BatchClass &c, int *blocks) {
-    if (c.mm) return pdit::mm_batch_blocks_per_sm(c.n, c.asym, blocks);
+    if (c.mm) return pdit::mm_batch_blocks_per_sm(c.n, c.form, blocks);
     if (c.dot) return pdit::dot_batch_blocks_per_sm(c.maxk, c.wpr, c.threads, c.smem, blocks);
     return c.asym ? batch_blocks_t<true>(c, blocks) : batch_blocks_t<false>(c, blocks);
 }
@@ -1602,7 +1613,7 @@ int batch_launch_t(const BatchClass &c, const pdit::SweepArgs *descs, int *queue
 }
 
 int batch_launch(const BatchClass &c, const pdit::SweepArgs *descs, int *queue) {
-    if (c.mm) return pdit::mm_batch_launch(c.n, c.asym, descs, c.d_units, c.nunits, queue, c.grid, c.stream);
+    if (c.mm) return pdit::mm_batch_launch(c.n, c.form, descs, c.d_units, c.nunits, queue, c.grid, c.stream);
     if (c.dot)
         return pdit::dot_batch_launch(c.maxk, c.wpr, descs, c.d_units, c.nunits, queue, c.grid, c.threads, c.smem,
                                       c.stream);
@@ -1611,7 +1622,7 @@ int batch_launch(const BatchClass &c, const pdit::SweepArgs *descs, int *queue) 
 
 // Same compiled kernel shape.
 bool same_class(const BatchClass &x, int dt, bool asym, const Plan &p) {
-    if (x.mm || p.mm) return x.mm == p.mm && x.asym == asym && x.maxk == p.maxk && x.lanes == p.lanes;
+    if (x.mm || p.mm) return x.mm == p.mm && x.form == p.form && x.maxk == p.maxk && x.lanes == p.lanes;
     if (x.dot || p.dot) return x.dot == p.dot && x.maxk == p.maxk && x.wpr == p.wpr;
     return x.dt == dt && x.asym == asym && x.maxk == p.maxk && x.wpr == p.wpr && x.pk == p.pk && x.tsmem == p.tsmem;
 }
@@ -1620,6 +1631,7 @@ bool same_class(const BatchClass &x, int dt, bool asym, const Plan &p) {
 BatchClass class_for(int dt, bool asym, const Plan &p, int n) {
     BatchClass x;
     x.mm = p.mm;
+    x.form = p.form;
     x.lanes = p.lanes;
     x.n = n;
     x.dt = dt;

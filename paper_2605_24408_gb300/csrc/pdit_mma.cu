@@ -1,6 +1,6 @@
 // Annealed p-dit sweep with the influence entries of many replicas formed by
-// tensor-core products (symmetric instances, zero diagonals, entries of D and
-// F in 0..127).
+// tensor-core products (zero diagonals; first: symmetric instances, entries
+// of D and F in 0..127).
 //
 // The two influence entries of Eq. 3 for the updating location i and each
 // candidate j (one-term table of Eq. 2, I[m][c] = sum_y D[m][y] F[c][p(y)])
@@ -31,6 +31,13 @@
 //   T[i][p(j)] = sum_c F[p(j)][c] D[i][p^-1(c)] + F[c][p(j)] D[p^-1(c)][i]:
 // the same products of twice the depth, [D | D^T] and [F | F^T] against
 // [q; q'] and [g; g']. A unit of energy is then 2^-48 itself.
+// Wide instances (symmetric, an entry above 127, none above 2047; N <= 128)
+// keep 16-bit tables, which read as f16 are their entries times 2^-24 too, and
+// split a vector's entries into their low 5 bits and the rest: two products
+// whose sums stay below 2^24 (N 2047 63), joined as int32; energies, h and the
+// swap are int32, states' energies 64 bits. N = 61, 512 replicas x 500 sweeps:
+// 24.3 ms (60.6 ms with the table kernels); 1.1 to 1.8 times their speed with
+// 64 replicas, 1.6 (N = 33) to 6.6 (N = 112) with 4096.
 //
 // Bound: the latency of an update's chain of about 450 instructions a warp
 // (issue slots 50% busy, 16 warps an SM at the register limit; shared-memory
@@ -41,15 +48,20 @@
 // kernels). Bytes instead of f16 words for the vectors, with h in registers,
 // cut the wavefronts by a fifth but were slower (2.03e9: more instructions);
 // products formed one location ahead by warps of their own were too (1.78e9).
+#include <type_traits>
+
 #include "pdit_f16.cuh"
 #include "pdit_sweep.cuh"
 
 namespace pdit {
 
-template <int K_, int LPR_, bool ASYM_ = false>
+template <int K_, int LPR_, int FORM_ = kMmSymmetric>
 struct MmShape {
-    static constexpr int K = K_, LPR = LPR_;
-    static constexpr bool ASYM = ASYM_;
+    static constexpr int K = K_, LPR = LPR_, FORM = FORM_;
+    static constexpr bool ASYM = FORM == kMmGeneral, WIDE = FORM == kMmWide;
+    using V = typename std::conditional<WIDE, int, float>::type;      // energies and influence entries
+    using E = typename std::conditional<WIDE, long long, int>::type;  // energies of states
+    static constexpr int ES = WIDE ? 2 : 1;       // bytes of a table entry
     static constexpr int NP = K * LPR;            // padded size
     static constexpr int MT = NP / 16;            // 16-row tiles of D and of F; 16-deep steps of a product
     static constexpr int NW = LPR == 16 ? 8 : 16; // warps per CTA
@@ -65,15 +77,16 @@ struct MmShape {
     // disjoint banks. Results, floats: 4 mod 16, so that the four column pairs
     // of a fragment store hit distinct banks and the two replicas of a warp,
     // 4 rows apart (crow), read disjoint ones.
-    static constexpr int DS = REGS ? 256 : 16 * (MT | 1);
     static constexpr int VS = 32 * (MT | 1);
+    static constexpr int DS = WIDE ? VS : REGS ? 256 : 16 * (MT | 1);
     static constexpr int CS = NP + 4;
     static constexpr int PS = 8 * LPR;            // permutation bytes of a replica (8 per thread)
     // shared memory (the tables first: their rows are 256-byte aligned)
     static constexpr int TT = NP * DS, VT = R * VS;  // from a table, a vector, to its transpose's
     static constexpr int NT2 = ASYM ? 2 : 1;      // the transposes after D and F, their vectors after q and g
-    static constexpr int oD = 0, oF = oD + NT2 * NP * DS, oVq = oF + NT2 * NP * DS, oVg = oVq + NT2 * R * VS,
-                         oC = oVg + NT2 * R * VS,
+    static constexpr int NV2 = ASYM || WIDE ? 2 : 1;  // (wide: the high parts after the low ones)
+    static constexpr int oD = 0, oF = oD + NT2 * NP * DS, oVq = oF + NT2 * NP * DS, oVg = oVq + NV2 * R * VS,
+                         oC = oVg + NV2 * R * VS,
                          oR = oC + 4 * R * CS, oH = oR + 4 * R * CS, oP = oH + 4 * R * CS, oI = oP + R * PS,
                          oDr = oI + R * PS, oX = oDr + 8 * NP, bytes = oX + 16;
     // result row of the replica in vector row v: bits 1 and 2 of v trade places
@@ -101,26 +114,50 @@ __device__ __forceinline__ int byte8(const uint2 v, int k) {
     return (int)__byte_perm(k < 4 ? v.x : v.y, 0, 0x4440 | (k & 3));
 }
 
-template <int K>
+__device__ __forceinline__ int lds_s32(uint32_t a) {
+    int v;
+    asm volatile("ld.shared.s32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ int lds_u16(uint32_t a) {
+    int v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+
+template <int K, typename V>
 struct MmVals {
-    float v[K];
+    V v[K];
 };
 
+// Weight of an outcome d above the least dmin: binary32 units of `scale`, or
+// integers of half the energy.
+__device__ __forceinline__ unsigned long long mm_weight(float d, float dmin, float scale, float beta) {
+    return eq5_weight_f((d - dmin) * scale, beta);
+}
+__device__ __forceinline__ unsigned long long mm_weight(int d, int dmin, float, float beta) {
+    return eq5_weight(2 * (d - dmin), beta);
+}
+__device__ __forceinline__ float mm_top(float) { return __int_as_float(0x7F800000); }
+__device__ __forceinline__ int mm_top(int) { return 0x7FFFFFFF; }
+__device__ __forceinline__ float mm_min(float a, float b) { return fminf(a, b); }
+__device__ __forceinline__ int mm_min(int a, int b) { return min(a, b); }
+
 // The exact draw (eq5_draw_exact) for one replica's LPR threads.
-template <int K, int LPR>
-__device__ __noinline__ int mm_exact_draw(const MmVals<K> d, int n, int t, float scale, float beta,
+template <int K, int LPR, typename V>
+__device__ __noinline__ int mm_exact_draw(const MmVals<K, V> d, int n, int t, float scale, float beta,
                                           unsigned long long draw, unsigned mask) {
-    float dmin = __int_as_float(0x7F800000);
+    V dmin = mm_top(V());
 #pragma unroll
     for (int k = 0; k < K; ++k)
-        if (t * K + k < n) dmin = fminf(dmin, d.v[k]);
+        if (t * K + k < n) dmin = mm_min(dmin, d.v[k]);
 #pragma unroll
-    for (int o = LPR / 2; o; o >>= 1) dmin = fminf(dmin, __shfl_xor_sync(mask, dmin, o, LPR));
+    for (int o = LPR / 2; o; o >>= 1) dmin = mm_min(dmin, __shfl_xor_sync(mask, dmin, o, LPR));
     unsigned long long pre[K];
     unsigned long long lsum = 0;
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-        if (t * K + k < n) lsum += eq5_weight_f((d.v[k] - dmin) * scale, beta);
+        if (t * K + k < n) lsum += mm_weight(d.v[k], dmin, scale, beta);
         pre[k] = lsum;
     }
     unsigned long long incl = lsum;
@@ -144,13 +181,33 @@ __device__ __noinline__ int mm_exact_draw(const MmVals<K> d, int n, int t, float
 // Address of entry byte8(v, k) of the table row at `row`.
 template <class S>
 __device__ __forceinline__ uint32_t entry(uint32_t row, const uint2 v, int k) {
-    if constexpr (S::DS == 256)
+    if constexpr (S::WIDE)
+        return row + 2u * (uint32_t)byte8(v, k);
+    else if constexpr (S::DS == 256)
         return __byte_perm(k < 4 ? v.x : v.y, row, 0x7650 | (k & 3));
     else
         return row + (uint32_t)byte8(v, k);
 }
 
-// D and F of an instance into the CTA's tables (bytes, zero outside n x n),
+// The table entry at an address.
+template <class S>
+__device__ __forceinline__ int lds_entry(uint32_t a) {
+    return S::WIDE ? lds_u16(a) : lds_u8(a);
+}
+
+// The fragment of a wide table: 16-bit entries are f16 numbers as they stand.
+template <int DS>
+__device__ __forceinline__ void mm_frag_wide(const uint8_t *tab, int row0, int s, int lane, uint32_t (&a)[4]) {
+    const uint8_t *p = tab + (row0 + (lane >> 2)) * DS + 32 * s + 8 * (lane & 3);
+    const uint2 x = *reinterpret_cast<const uint2 *>(p);
+    const uint2 y = *reinterpret_cast<const uint2 *>(p + 8 * DS);
+    a[0] = x.x;
+    a[1] = y.x;
+    a[2] = x.y;
+    a[3] = y.y;
+}
+
+// D and F of an instance into the CTA's tables (zero outside n x n),
 // and the warp's rows into registers where they stay there. Ends with the
 // CTA synchronised.
 template <class S>
@@ -161,6 +218,11 @@ __device__ __forceinline__ void mm_stage(const int32_t *D, const int32_t *F, int
     __syncthreads();
     for (int idx = threadIdx.x; idx < n * n; idx += S::T) {
         const int x = idx / n, y = idx - x * n;
+        if constexpr (S::WIDE) {
+            *reinterpret_cast<uint16_t *>(sm + S::oD + S::loc(x) * S::DS + 2 * S::loc(y)) = (uint16_t)D[idx];
+            *reinterpret_cast<uint16_t *>(sm + S::oF + x * S::DS + 2 * y) = (uint16_t)F[idx];
+            continue;
+        }
         sm[S::oD + S::loc(x) * S::DS + S::loc(y)] = (uint8_t)D[idx];
         sm[S::oF + x * S::DS + y] = (uint8_t)F[idx];
         if constexpr (S::ASYM) {
@@ -176,7 +238,12 @@ __device__ __forceinline__ void mm_stage(const int32_t *D, const int32_t *F, int
         for (int jt = 0; jt < S::JT; ++jt) {
             const int m = min(w % (S::NW / 2) + jt * (S::NW / 2), S::MT - 1);
 #pragma unroll
-            for (int s = 0; s < S::MT; ++s) mm_frag<S::DS>(tab, 16 * m, s, threadIdx.x & 31, A[jt][s]);
+            for (int s = 0; s < S::MT; ++s) {
+                if constexpr (S::WIDE)
+                    mm_frag_wide<S::DS>(tab, 16 * m, s, threadIdx.x & 31, A[jt][s]);
+                else
+                    mm_frag<S::DS>(tab, 16 * m, s, threadIdx.x & 31, A[jt][s]);
+            }
         }
     }
 }
@@ -191,27 +258,28 @@ __device__ __forceinline__ void mm_products(unsigned char *sm, int w, const uint
     if (m0 >= S::MT) return;
     const uint8_t *tab = sm + (second ? S::oF : S::oD);
     const unsigned char *v = sm + (second ? S::oVg : S::oVq) + g * S::VS + 8 * q;
-    float acc[S::JT][NT][4];
+    constexpr int NA = S::WIDE ? 2 : 1;  // wide: the high parts' products by themselves
+    float acc[S::JT][NA * NT][4];
 #pragma unroll
     for (int jt = 0; jt < S::JT; ++jt)
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
+        for (int nt = 0; nt < NA * NT; ++nt)
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc[jt][nt][e] = 0.0f;
 #pragma unroll
     for (int d = 0; d < S::NT2 * S::MT; ++d) {
         const int s = d % S::MT, tr = d / S::MT;  // the second half: the transposes
-        uint2 b[NT];
+        uint2 b[NA * NT];
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-            b[nt] = *reinterpret_cast<const uint2 *>(v + tr * S::VT + 8 * nt * S::VS + 32 * s);
+        for (int nt = 0; nt < NA * NT; ++nt)
+            b[nt] = *reinterpret_cast<const uint2 *>(v + (tr + nt / NT) * S::VT + 8 * (nt % NT) * S::VS + 32 * s);
 #pragma unroll
         for (int jt = 0; jt < S::JT; ++jt) {
             const int m = m0 + jt * (S::NW / 2);
             if (S::MT % (S::NW / 2) != 0 && jt == S::JT - 1 && m >= S::MT) continue;
             if constexpr (S::REGS) {
 #pragma unroll
-                for (int nt = 0; nt < NT; ++nt) mma_f16(acc[jt][nt], A[jt][s], b[nt]);
+                for (int nt = 0; nt < NA * NT; ++nt) mma_f16(acc[jt][nt], A[jt][s], b[nt]);
             } else {
                 uint32_t a[4];
                 mm_frag<S::DS>(tab + tr * S::TT, 16 * m, s, lane, a);
@@ -221,18 +289,27 @@ __device__ __forceinline__ void mm_products(unsigned char *sm, int w, const uint
         }
     }
     // columns 2q and 2q + 1 of a tile go to result rows crow(2q) and, one on, crow(2q + 1)
-    float *out = reinterpret_cast<float *>(sm + (second ? S::oR : S::oC)) + S::crow(2 * q) * S::CS + g;
+    using V = typename S::V;
+    V *out = reinterpret_cast<V *>(sm + (second ? S::oR : S::oC)) + S::crow(2 * q) * S::CS + g;
 #pragma unroll
     for (int jt = 0; jt < S::JT; ++jt) {
         const int m = m0 + jt * (S::NW / 2);
         if (m >= S::MT) break;
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
-            float *o = out + 8 * nt * S::CS + 16 * m;
-            o[0] = acc[jt][nt][0];
-            o[S::CS] = acc[jt][nt][1];
-            o[8] = acc[jt][nt][2];
-            o[S::CS + 8] = acc[jt][nt][3];
+            V *o = out + 8 * nt * S::CS + 16 * m;
+            V x[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                if constexpr (S::WIDE)  // units of 2^-48: low + 32 high
+                    x[e] = (int)(acc[jt][nt][e] * (0.5f * kMmScale)) + 32 * (int)(acc[jt][NT + nt][e] * (0.5f * kMmScale));
+                else
+                    x[e] = acc[jt][nt][e];
+            }
+            o[0] = x[0];
+            o[S::CS] = x[1];
+            o[8] = x[2];
+            o[S::CS + 8] = x[3];
         }
     }
 }
@@ -254,14 +331,18 @@ __device__ __forceinline__ void mm_diagonal(const unsigned char *sm, const uint8
         const uint8_t *dr = sm + S::oD + S::loc(y) * S::DS, *fr = sm + S::oF + pb[S::pbyte(y)] * S::DS;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
-            h[k] += (int)dr[S::pos(t, k)] * (int)fr[px[k]];
+            if constexpr (S::WIDE)
+                h[k] += (int)reinterpret_cast<const uint16_t *>(dr)[S::pos(t, k)] *
+                        (int)reinterpret_cast<const uint16_t *>(fr)[px[k]];
+            else
+                h[k] += (int)dr[S::pos(t, k)] * (int)fr[px[k]];
             if constexpr (S::ASYM) h[k] += (int)dr[S::TT + S::pos(t, k)] * (int)fr[S::TT + px[k]];
         }
     }
 }
 
-template <int LPR>
-__device__ __forceinline__ int mm_sum(int v, unsigned mask) {
+template <int LPR, typename E>
+__device__ __forceinline__ E mm_sum(E v, unsigned mask) {
 #pragma unroll
     for (int o = LPR / 2; o; o >>= 1) v += __shfl_xor_sync(mask, v, o, LPR);
     return v;
@@ -273,7 +354,9 @@ template <class S>
 __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int part, unsigned char *sm,
                                              const uint32_t (&A)[S::JT][S::REGS ? S::MT : 1][4]) {
     constexpr int K = S::K, LPR = S::LPR;
-    constexpr bool ASYM = S::ASYM;
+    constexpr bool ASYM = S::ASYM, WIDE = S::WIDE;
+    using V = typename S::V;
+    using Acc = typename S::E;
     constexpr float kScale = ASYM ? 0.5f * kMmScale : kMmScale;
     const int tid = threadIdx.x, w = __shfl_sync(kFull, tid >> 5, 0), lane = tid & 31;
     const int half = LPR == 16 ? lane >> 4 : 0;
@@ -290,9 +373,9 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
     const bool warp_live = (LPR == 16 && count > 8 ? 2 * w : v0) < count;
     const int r = r0 + idx;
     const uint32_t grep = a.rep_base + (uint32_t)r;
-    float *sC = reinterpret_cast<float *>(sm + S::oC) + S::crow(slot) * S::CS;
-    float *sR = reinterpret_cast<float *>(sm + S::oR) + S::crow(slot) * S::CS;
-    float *sH = reinterpret_cast<float *>(sm + S::oH) + S::crow(slot) * S::CS;
+    V *sC = reinterpret_cast<V *>(sm + S::oC) + S::crow(slot) * S::CS;
+    V *sR = reinterpret_cast<V *>(sm + S::oR) + S::crow(slot) * S::CS;
+    V *sH = reinterpret_cast<V *>(sm + S::oH) + S::crow(slot) * S::CS;
     uint8_t *pb = sm + S::oP + slot * S::PS;
     uint8_t *ib = sm + S::oI + slot * S::PS;
     float *drow = reinterpret_cast<float *>(sm + S::oDr);
@@ -305,9 +388,10 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
     int32_t *gbp = a.best_perm + (size_t)r * n;
     const bool fresh = part == 0 && a.fresh;
 
-    // (|E| <= n^2 127^2 < 2^31, and twice that in the general form's sums)
+    // (|E| <= n^2 127^2 < 2^31, and twice that in the general form's sums;
+    // wide: 64 bits)
     // (the best sweep and the accepted swaps stay in global memory)
-    int E = 0, bestE = 0;
+    Acc E = 0, bestE = 0;
     bool reached = false;
     if (warp_live) {
         // ---- permutation: bytes by thread, and its inverse. A slot without
@@ -346,13 +430,17 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
         }
         __syncwarp();
         // ---- p-diagonal and energy: E = sum_x h[x] (Eq. 1 regrouped)
-        int h[K], esum = 0;
+        int h[K];
+        Acc esum = 0;
         mm_diagonal<S>(sm, pb, n, t, h);
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             esum += h[k];
             // an entry beyond n: an energy of +infinity, a weight of 0
-            sH[S::pos(t, k)] = t * K + k < n ? (float)h[k] * kMmUnit : __int_as_float(0xFF800000);
+            if constexpr (WIDE)
+                sH[S::pos(t, k)] = h[k];
+            else
+                sH[S::pos(t, k)] = t * K + k < n ? (float)h[k] * kMmUnit : __int_as_float(0xFF800000);
         }
         esum = mm_sum<LPR>(esum, kFull);
         if constexpr (S::ASYM) esum >>= 1;
@@ -366,8 +454,8 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
                     note_target(a, bestE, -1, reached);
                 }
             } else {
-                E = (int)__ldcg(a.energy + r);
-                bestE = (int)__ldcg(a.best_energy + r);
+                E = (Acc)__ldcg(a.energy + r);
+                bestE = (Acc)__ldcg(a.best_energy + r);
                 if (E != esum && t == 0) atomicOr(a.status, 1);
             }
         }
@@ -390,7 +478,7 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
             if (*flag) break;
         }
         // (never 0, so that an infinite energy always has weight 0)
-        const float kb = fminf(-beta_of(s) * kLog2e * kScale, -1e-37f);
+        const float kb = fminf(-beta_of(s) * kLog2e * (WIDE ? 2.0f : kScale), -1e-37f);
         uint32_t rhi = 0;  // high words of the draws of LPR locations
         int moves = 0;
         // location i = ti K + ki
@@ -406,7 +494,9 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
             int pi = 0, qb[K], qt[ASYM ? K : 1];  // F_ab, F_ba of this thread's locations
             uint32_t aFi = 0;
             // ---- vectors
-            if (tid < S::NP) {
+            if constexpr (WIDE) {
+                if (tid < S::NP) asm volatile("st.shared.b32 [%0], %1;" ::"r"(aDr + 4 * tid), "r"(2 * lds_u16(aDi + 2 * tid)));
+            } else if (tid < S::NP) {
                 const float x = ASYM ? (float)(lds_u8(aDi + tid) + lds_u8(aDi + S::TT + tid)) * kMmUnit
                                      : (float)lds_u8(aDi + tid) * (2.0f * kMmUnit);
                 asm volatile("st.shared.f32 [%0], %1;" ::"r"(aDr + 4 * tid), "f"(x));
@@ -418,17 +508,24 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
                 aFi = base32 + S::oF + pi * S::DS;
                 auto put = [&](uint32_t at, const int (&x)[K]) {
 #pragma unroll
-                    for (int k = 0; k + 1 < K; k += 2)
-                        asm volatile("st.shared.b32 [%0], %1;" ::"r"(at + k * 2 * LPR),
-                                     "r"(__byte_perm(x[k], x[k + 1], 0x5410)));
-                    if constexpr (K & 1)
-                        asm volatile("st.shared.b16 [%0], %1;" ::"r"(at - 2 * t + (K - 1) * 2 * LPR), "h"((uint16_t)x[K - 1]));
+                    for (int k = 0; k < K; k += 2) {
+                        const uint32_t v = k + 1 < K ? __byte_perm(x[k], x[k + 1 < K ? k + 1 : k], 0x5410) : (uint32_t)x[k];
+#pragma unroll
+                        for (int part = 0; part < (WIDE ? 2 : 1); ++part) {  // low 5 bits, the bits above
+                            const uint32_t y = !WIDE ? v : part == 0 ? v & 0x001F001Fu : (v >> 5) & 0x003F003Fu;
+                            if (k + 1 < K)
+                                asm volatile("st.shared.b32 [%0], %1;" ::"r"(at + part * S::VT + k * 2 * LPR), "r"(y));
+                            else
+                                asm volatile("st.shared.b16 [%0], %1;" ::"r"(at + part * S::VT - 2 * t + k * 2 * LPR),
+                                             "h"((uint16_t)y));
+                        }
+                    }
                 };
                 int gb[K];
 #pragma unroll
-                for (int k = 0; k < K; ++k) gb[k] = lds_u8(entry<S>(aDi, i8, k));
+                for (int k = 0; k < K; ++k) gb[k] = lds_entry<S>(entry<S>(aDi, i8, k));
 #pragma unroll
-                for (int k = 0; k < K; ++k) qb[k] = lds_u8(entry<S>(aFi, p8, k));
+                for (int k = 0; k < K; ++k) qb[k] = lds_entry<S>(entry<S>(aFi, p8, k));
                 put(aV + (S::oVg - S::oVq), gb);
                 put(aV, qb);
                 if constexpr (ASYM) {
@@ -450,9 +547,22 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
             if (warp_live) {
                 // ---- swap energies, half of Eq. 3, up to the common h_i:
                 // I[i][p(j)] + I[j][p(i)] - h_j + 2 D_ij F_ab
-                const float hi = lds_f32(aR + 4 * pi);  // I[i][p(i)]
-                MmVals<K> e;
-                float hk[K], mq[K];
+                V hi;  // I[i][p(i)]
+                MmVals<K, V> e;
+                V hk[K];
+                float mq[WIDE ? 1 : K], pre[K], lsum = 0.0f;
+                if constexpr (WIDE) {
+                    hi = lds_s32(aR + 4 * pi);
+#pragma unroll
+                    for (int k = 0; k < K; ++k) {
+                        const uint32_t x = 4 * S::pos(t, k);
+                        hk[k] = lds_s32(aH + x);
+                        e.v[k] = lds_s32(aDr + x) * qb[k] + lds_s32(aR + 4 * byte8(p8, k)) + (lds_s32(aC + x) - hk[k]);
+                        const float w = ex2_approx(__int2float_rn(e.v[k] - hi) * kb);
+                        pre[k] = t * K + k < n ? w : 0.0f;
+                    }
+                } else {
+                hi = lds_f32(aR + 4 * pi);
 #pragma unroll
                 for (int k = 0; k < K; ++k)  // 2^23 + F_ab (F_ab + F_ba)
                     mq[k] = __int_as_float(0x4B000000 | (ASYM ? qb[k] + qt[ASYM ? k : 0] : qb[k]));
@@ -479,7 +589,6 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
                 // ---- binary32 draw, kept where it is certainly the exact
                 // one (eq5_draw_core): no interval end within m of t
                 const float bias = -kb * hi;
-                float pre[K], lsum = 0.0f;
 #pragma unroll
                 for (int k = 0; k + 1 < K; k += 2) {
                     const float2 x = fma2(make_float2(e.v[k], e.v[k + 1]), two(kb), two(bias));
@@ -487,6 +596,7 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
                     pre[k + 1] = ex2_approx(x.y);
                 }
                 if constexpr (K & 1) pre[K - 1] = ex2_approx(fmaf(e.v[K - 1], kb, bias));
+                }
 #pragma unroll
                 for (int k = 0; k < K; ++k) {
                     lsum += pre[k];
@@ -529,9 +639,24 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
                     const int fb = (v >> 16) & 0xFF;
                     const int xj = S::pos(tj, kj);
                     const uint32_t aFj = base32 + S::oF + fb * S::DS, aDj = base32 + S::oD + xj * S::DS;
-                    const float rs = lds_f32(aR + 4 * fb), cs = lds_f32(aC + 4 * xj), hs = lds_f32(aH + 4 * xj);
-                    // what the swap adds to both moved entries of h: D_ij F_ab (D_ij F_ba + D_ji F_ab)
-                    float dq, dd;
+                    V rs, cs, dq, dd;  // dq: what the swap adds to both moved entries of h, D_ij F_ab (D_ij F_ba + D_ji F_ab)
+                    V hw[WIDE ? K : 1];
+                    float2 hn[WIDE ? 1 : K / 2 + 1];
+                    if constexpr (WIDE) {
+                        rs = lds_s32(aR + 4 * fb);
+                        cs = lds_s32(aC + 4 * xj);
+                        dq = (lds_s32(aDr + 4 * xj) >> 1) * lds_u16(aFi + 2 * fb);
+                        dd = (rs - hi) + (cs - lds_s32(aH + 4 * xj)) + 2 * dq;
+                        // h[m] += (D_im - D_jm) (F_b,p(m) - F_a,p(m))
+#pragma unroll
+                        for (int k = 0; k < K; ++k) {
+                            const int u = (lds_s32(aDr + 4 * S::pos(t, k)) >> 1) - lds_u16(aDj + 2 * S::pos(t, k));
+                            hw[k] = hk[k] + u * (lds_u16(entry<S>(aFj, p8, k)) - qb[k]);
+                        }
+                    } else {
+                    rs = lds_f32(aR + 4 * fb);
+                    cs = lds_f32(aC + 4 * xj);
+                    const float hs = lds_f32(aH + 4 * xj);
                     if constexpr (ASYM) {
                         const int fab = lds_u8(aFi + fb), fba = lds_u8(aFi + S::TT + fb);
                         dq = (float)(lds_u8(aDi + xj) * fba + lds_u8(aDi + S::TT + xj) * fab) * kMmUnit;
@@ -540,8 +665,8 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
                         dq = 0.5f * lds_f32(aDr + 4 * xj) * (float)lds_u8(aFi + fb);
                         dd = 2.0f * dq;
                     }
+                    dd = (rs - hi) + (cs - hs) + dd;
                     // h[m] += (D_im - D_jm) (F_b,p(m) - F_a,p(m))
-                    float2 hn[K / 2 + 1];
                     auto word = [&](uint32_t at) {  // a pair of a row of D at this thread's locations
                         uint32_t x;
                         asm volatile("ld.shared.u16 %0, [%1];" : "=r"(x) : "r"(at + 2 * t));
@@ -581,12 +706,19 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
                                      ones(lds_u8(entry<S>(aFj, p8, k) + S::TT)) - ones(qt[k]), x);
                         hn[K / 2].x = x;
                     }
+                    }
                     __syncwarp();  // reads of h and p by the replica's threads done
                     if (sw) {
+                        if constexpr (WIDE) {
+#pragma unroll
+                            for (int k = 0; k < K; ++k) sH[S::pos(t, k)] = hw[k];
+                            E += 2 * dd;
+                        } else {
 #pragma unroll
                         for (int k = 0; k + 1 < K; k += 2) *reinterpret_cast<float2 *>(sH + k * LPR + 2 * t) = hn[k / 2];
                         if constexpr (K & 1) sH[(K - 1) * LPR + t] = hn[K / 2].x;
-                        E += (int)(((rs - hi) + (cs - hs) + dd) * kScale);
+                        E += (int)(dd * kScale);
+                        }
                         moves += 1;
                     }
                     __syncwarp();
@@ -625,7 +757,8 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
     // back
     if (warp_live) {
         if (a.audit && part >= a.segments - 1) {
-            int h[K], eq1 = 0;
+            int h[K];
+            Acc eq1 = 0;
             mm_diagonal<S>(sm, pb, n, t, h);
 #pragma unroll
             for (int k = 0; k < K; ++k) eq1 += h[k];
@@ -719,9 +852,9 @@ struct MmCall {
     int *batch_blocks = nullptr;
 };
 
-template <int K, int LPR, bool ASYM>
+template <int K, int LPR, int FORM>
 static int mm_one(const MmCall &c) {
-    using S = MmShape<K, LPR, ASYM>;
+    using S = MmShape<K, LPR, FORM>;
     const bool batch = c.descs || c.batch_blocks;
     const cudaError_t e =
         batch ? cudaFuncSetAttribute(mm_batch_kernel<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::bytes)
@@ -744,55 +877,58 @@ static int mm_one(const MmCall &c) {
     return (int)cudaGetLastError();
 }
 
-template <bool ASYM>
+template <int FORM>
 static int mm_dispatch_form(int n, const MmCall &c) {
     if (n <= 128) {
         switch ((n + 15) / 16) {
-        case 3: return mm_one<3, 16, ASYM>(c);
-        case 4: return mm_one<4, 16, ASYM>(c);
-        case 5: return mm_one<5, 16, ASYM>(c);
-        case 6: return mm_one<6, 16, ASYM>(c);
-        case 7: return mm_one<7, 16, ASYM>(c);
-        default: return mm_one<8, 16, ASYM>(c);
+        case 3: return mm_one<3, 16, FORM>(c);
+        case 4: return mm_one<4, 16, FORM>(c);
+        case 5: return mm_one<5, 16, FORM>(c);
+        case 6: return mm_one<6, 16, FORM>(c);
+        case 7: return mm_one<7, 16, FORM>(c);
+        default: return mm_one<8, 16, FORM>(c);
         }
     }
-    if ((n + 31) / 32 == 5) return mm_one<5, 32, ASYM>(c);
-    if constexpr (!ASYM) {  // (the general form's four tables end at 160 locations)
+    if constexpr (FORM != kMmWide)
+        if ((n + 31) / 32 == 5) return mm_one<5, 32, FORM>(c);
+    if constexpr (FORM == kMmSymmetric) {  // (the general form's four tables end at 160 locations)
         switch ((n + 31) / 32) {
-        case 6: return mm_one<6, 32, ASYM>(c);
-        case 7: return mm_one<7, 32, ASYM>(c);
-        default: return mm_one<8, 32, ASYM>(c);
+        case 6: return mm_one<6, 32, FORM>(c);
+        case 7: return mm_one<7, 32, FORM>(c);
+        default: return mm_one<8, 32, FORM>(c);
         }
     }
     return (int)cudaErrorInvalidValue;
 }
 
-static int mm_dispatch(int n, bool asym, const MmCall &c) {
-    if (n <= 32 || n > (asym ? kMmGeneralMax : 256)) return (int)cudaErrorInvalidValue;
-    return asym ? mm_dispatch_form<true>(n, c) : mm_dispatch_form<false>(n, c);
+static int mm_dispatch(int n, int form, const MmCall &c) {
+    if (n <= 32 || n > kMmMax[form]) return (int)cudaErrorInvalidValue;
+    return form == kMmGeneral ? mm_dispatch_form<kMmGeneral>(n, c)
+         : form == kMmWide    ? mm_dispatch_form<kMmWide>(n, c)
+                              : mm_dispatch_form<kMmSymmetric>(n, c);
 }
 
-int mm_query(int n, bool asym, MmInfo *info) {
+int mm_query(int n, int form, MmInfo *info) {
     MmCall c;
     c.info = info;
-    return mm_dispatch(n, asym, c);
+    return mm_dispatch(n, form, c);
 }
 
-int mm_launch(const SweepArgs &a, bool asym, int grid, cudaStream_t st) {
+int mm_launch(const SweepArgs &a, int form, int grid, cudaStream_t st) {
     MmCall c;
     c.args = &a;
     c.grid = grid;
     c.st = st;
-    return mm_dispatch(a.n, asym, c);
+    return mm_dispatch(a.n, form, c);
 }
 
-int mm_batch_blocks_per_sm(int n, bool asym, int *blocks) {
+int mm_batch_blocks_per_sm(int n, int form, int *blocks) {
     MmCall c;
     c.batch_blocks = blocks;
-    return mm_dispatch(n, asym, c);
+    return mm_dispatch(n, form, c);
 }
 
-int mm_batch_launch(int n, bool asym, const SweepArgs *descs, const BatchUnit *units, int nunits, int *queue, int grid,
+int mm_batch_launch(int n, int form, const SweepArgs *descs, const BatchUnit *units, int nunits, int *queue, int grid,
                     cudaStream_t st) {
     MmCall c;
     c.descs = descs;
@@ -801,7 +937,7 @@ int mm_batch_launch(int n, bool asym, const SweepArgs *descs, const BatchUnit *u
     c.queue = queue;
     c.grid = grid;
     c.st = st;
-    return mm_dispatch(n, asym, c);
+    return mm_dispatch(n, form, c);
 }
 
 }  // namespace pdit

@@ -1746,18 +1746,21 @@ int small_query(int n, bool f32, int warps, SmallInfo *info);
 int small_launch(const SweepArgs &a, bool f32, int grid, int warps, cudaStream_t stream);
 
 // Tensor-core product kernel (pdit_mma.cu): zero diagonals and entries in
-// 0..127, symmetric or (up to kMmGeneralMax locations) general; one compiled
-// kernel per range of n.
+// 0..127 (symmetric: 0..2047); one compiled kernel per form and range of n.
 // Return a cudaError_t value.
 struct MmInfo {
     int threads, slots, lanes, k, blocks_per_sm;  // slots: replicas per CTA; lanes: threads per replica
     size_t smem;
 };
-constexpr int kMmGeneralMax = 160;
-int mm_query(int n, bool asym, MmInfo *info);
-int mm_launch(const SweepArgs &a, bool asym, int grid, cudaStream_t stream);
-int mm_batch_blocks_per_sm(int n, bool asym, int *blocks);
-int mm_batch_launch(int n, bool asym, const SweepArgs *descs, const BatchUnit *units, int nunits, int *queue, int grid,
+// Forms: symmetric and general with entries in 0..127, symmetric with entries
+// in 0..kMmWideTop; the largest sizes.
+constexpr int kMmSymmetric = 0, kMmGeneral = 1, kMmWide = 2;
+constexpr int kMmMax[3] = {256, 160, 128};
+constexpr int kMmWideTop = 2047;
+int mm_query(int n, int form, MmInfo *info);
+int mm_launch(const SweepArgs &a, int form, int grid, cudaStream_t stream);
+int mm_batch_blocks_per_sm(int n, int form, int *blocks);
+int mm_batch_launch(int n, int form, const SweepArgs *descs, const BatchUnit *units, int nunits, int *queue, int grid,
                     cudaStream_t stream);
 
 // Concurrent-update kernel (pdit_concurrent.cu): mode 3 of symmetric instances
