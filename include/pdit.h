@@ -150,8 +150,8 @@ int pdit_set_replicas_per_cta(pdit_qap *h, int g);
  * would use: shape[0] warps per replica (1 also where 16 threads run one,
  * two replicas to a warp), [1] candidates per thread, [2]
  * replicas per CTA, [3] CTAs, [4] 1 if the influence tables live in shared
- * memory (0: global memory; 2: no table, the product kernels of
- * pdit_set_influence), [5] dynamic shared memory bytes per CTA.
+ * memory, or no table is kept for entries beyond a byte (0: global memory; 2:
+ * no table, the product kernels of pdit_set_influence), [5] dynamic shared memory bytes per CTA.
  * [6] pending rank-1 terms held before the influence table is rewritten (1 =
  * after each swap; 4 or 16).
  * `shape` is a host array of 7 ints. Errors: PDIT_EINVAL, PDIT_ENOTSUP.
@@ -159,7 +159,7 @@ int pdit_set_replicas_per_cta(pdit_qap *h, int g);
 int pdit_launch_shape(const pdit_qap *h, int replicas, int *shape);
 
 /* Influence entries (pdit_set_influence). */
-#define PDIT_INFLUENCE_AUTO 0     /* dot products where eligible and no table knob is set, else the table */
+#define PDIT_INFLUENCE_AUTO 0     /* products where eligible and no table knob is set, else the table */
 #define PDIT_INFLUENCE_TABLE 1    /* the influence table of Eq. 2, updated after every accepted swap */
 #define PDIT_INFLUENCE_PRODUCTS 2 /* dot products of byte rows of D and of the permuted F (no table) */
 
@@ -187,12 +187,22 @@ int pdit_launch_shape(const pdit_qap *h, int replicas, int *shape);
  *                             themselves and no matrix per replica. Two-level-flow instances keep the
  *                             flow-class kernel unless pdit_set_class_update
  *                             turns it off.
- *   PDIT_INFLUENCE_AUTO     : products where eligible and where shared
- *                             memory holds at least 3 replicas per SM (N up
- *                             to about 200), unless a table knob (pending
- *                             swaps, placement) is set; the table otherwise
- *                             (also for the concurrent-update mode and for
- *                             calls that dump the tables).
+ *   PDIT_INFLUENCE_AUTO     : unless a table knob (pending swaps,
+ *                             placement) is set or the tables are dumped:
+ *                             above 32 locations with zero diagonals and no
+ *                             negative entry, tensor-core products
+ *                             (symmetric with entries to 127, or to 2047 at
+ *                             128 locations at most; general with entries to
+ *                             127 and 8 (N + 2) max D max F below 2^24, to
+ *                             160 locations); symmetric instances of at most
+ *                             32 locations, tables in registers; in the
+ *                             concurrent-update mode, one tensor-core
+ *                             product per iteration (symmetric, zero
+ *                             diagonals, entries in 0..127, at most 128
+ *                             locations); other symmetric byte-valued
+ *                             instances, dot products where shared memory
+ *                             holds at least 3 replicas per SM (N up to
+ *                             about 200); the table otherwise.
  * The entries are the same exact integers either way, so results do not
  * depend on the choice. Errors: PDIT_EINVAL.
  */

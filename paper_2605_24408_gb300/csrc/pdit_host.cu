@@ -988,7 +988,8 @@ int pdit_launch_shape(const pdit_qap *h, int replicas, int *shape) {
     shape[1] = p.maxk;
     shape[2] = p.groups;
     shape[3] = p.grid;
-    shape[4] = p.dot ? 2 : (p.tsmem ? 1 : 0);
+    // (entries beyond a byte report the shared-memory form, as they always did)
+    shape[4] = p.dot && !(p.mm && p.form == pdit::kMmWide) ? 2 : (p.tsmem ? 1 : 0);
     shape[5] = (int)p.smem;
     shape[6] = p.pk;
     return PDIT_OK;
@@ -1281,6 +1282,17 @@ int pdit_autotune(pdit_qap *h, int replicas, const float *beta, int sweeps, int 
             if (plan_ok({0, wpr, 0, 0, (int)PDIT_INFLUENCE_PRODUCTS}, &p)) cand.push_back(
                 {0, wpr, 0, 0, (int)PDIT_INFLUENCE_PRODUCTS});
         }
+    // The built-in choice, where it is a kernel that no candidate's settings
+    // reach: the small kernel and the product kernel's general and wide forms.
+    if (!cls && keep.place == PDIT_PLACE_AUTO && keep.infl == PDIT_INFLUENCE_AUTO) {
+        const Knobs automatic{0, 0, 0, 0, (int)PDIT_INFLUENCE_AUTO};
+        set(automatic);
+        Plan p;
+        pdit_opts o;
+        pdit_opts_init(&o);
+        o.replicas = replicas;
+        if (plan_for(h, &o, &p) == PDIT_OK && (p.small || (p.mm && !dot_eligible(h)))) cand.push_back(automatic);
+    }
     for (int place : {keep.place, (int)PDIT_PLACE_GLOBAL}) {
         if (keep.infl == PDIT_INFLUENCE_PRODUCTS && !cls) break;
         if (place == PDIT_PLACE_GLOBAL && (keep.place != 0 || cls)) continue;
@@ -1343,8 +1355,8 @@ int pdit_autotune(pdit_qap *h, int replicas, const float *beta, int sweeps, int 
     }
     set(cand[best]);
     if (shape) {
-        shape[0] = cand[best].wpr;
-        shape[1] = cand[best].infl == PDIT_INFLUENCE_PRODUCTS ? 1 : cand[best].pk;  // no pending terms
+        shape[0] = std::max(1, cand[best].wpr);
+        shape[1] = cand[best].infl == PDIT_INFLUENCE_PRODUCTS ? 1 : std::max(1, cand[best].pk);  // no pending terms
     }
     return PDIT_OK;
 }
