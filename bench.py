@@ -63,12 +63,12 @@ WORKLOAD_TEXT = {
 METRIC = "p-dit updates/s"
 L2_FLUSH_BYTES = 512 << 20
 SMEM_BYTES_PER_CLK = 128  # shared-memory bandwidth per SM per clock (32 banks x 4 B)
-TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dot_kernel_n100_traffic.json")
+TRAFFIC_FILE = os.path.join(ROOT, "profiles", "mm_kernel_n100_traffic.json")
 # the n100 kernel's own sources; the stored DRAM counters also record the
 # kernel and the launch shape they were taken with, and all must match to be
 # reported
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_2605_24408_gb300", "csrc", f)
-                  for f in ("pdit_sweep.cuh", "pdit_dot.cu")]
+                  for f in ("pdit_sweep.cuh", "pdit_f16.cuh", "pdit_mma.cu")]
 
 
 def kernel_source_sha() -> str:
@@ -98,6 +98,49 @@ def dot_kernel_name(maxk: int, wpr: int, n: int, parts: int = 1) -> str:
     fourth is 1 for a call split into parts."""
     nch = 7 if (maxk, wpr) == (4, 1) and product_stride(n) == 16 * 7 else 0
     return "dot_kernel<%d,%d,%d,%d>" % (maxk, wpr, nch, 1 if parts > 1 else 0)
+
+
+def mm_shape(n: int):
+    """(locations per thread, threads per replica, padded size) of the
+    tensor-core product kernel at size n."""
+    lanes = 16 if n <= 128 else 32
+    k = -(-n // lanes)
+    return k, lanes, k * lanes
+
+
+def mm_form(n: int, top: int, general: bool, nonneg_zero_diag: bool):
+    """The tensor-core product kernel's form that an instance runs, None where
+    it is not eligible (the library's rule)."""
+    if not nonneg_zero_diag or n <= 32:
+        return None
+    if general:
+        return "general" if top <= 127 and n <= 160 and 8 * (n + 2) * top * top < 1 << 24 else None
+    return "symmetric" if top <= 127 else "wide" if top <= 2047 and n <= 128 else None
+
+
+def mm_bytes_per_update(n: int, accept_frac: float, form: str) -> float:
+    """Shared-memory bytes one update moves in the tensor-core product kernel
+    (NP the padded size): per operand the two gathers (N entries) and the
+    vectors written (2 NP each) and read by half of the CTA's warps (4 or 8 of
+    them, 2 NP each), the two result vectors and the scaled row of D written
+    (4 NP each) and read, h and p read; per accepted swap an F row, a D row and
+    the scaled D row read and h written. The general and the wide form have
+    two vectors in each one's place."""
+    k, lanes, NP = mm_shape(n)
+    e = 2 if form == "wide" else 1
+    vec = 1 if form == "symmetric" else 2
+    warps = 4 if lanes == 16 else 8
+    swap = (e * (2 if form == "general" else 1)) * 2 * n + 8 * NP
+    gathers = 2 * n * (2 if form == "general" else e)
+    return gathers + 2 * vec * 2 * NP * (1 + warps) + 3 * 8 * NP + 6 * NP + accept_frac * swap
+
+
+def mm_macs_per_update(n: int, form: str) -> int:
+    """Tensor-core multiply-adds per update: two padded matrix-vector
+    products; twice that in the general form (both transposes) and the wide
+    one (both parts of a vector)."""
+    NP = mm_shape(n)[2]
+    return 2 * NP * NP * (1 if form == "symmetric" else 2)
 
 
 def host_cores() -> int:
@@ -688,8 +731,16 @@ def main():
         P.pdit_set_table_placement(q, args.place)
     infl = {"auto": P.PDIT_INFLUENCE_AUTO, "table": P.PDIT_INFLUENCE_TABLE,
             "products": P.PDIT_INFLUENCE_PRODUCTS}[args.influence]
-    if args.mode == "cupim" and infl == P.PDIT_INFLUENCE_AUTO:
-        infl = P.PDIT_INFLUENCE_TABLE  # concurrent updates run the table kernels: report their shape
+    top = int(max(np.abs(D).max(), np.abs(F).max()))
+    plain = bool(D.min() >= 0 and F.min() >= 0 and not D.diagonal().any() and not F.diagonal().any())
+    symmetric = bool(np.array_equal(D, D.T) and np.array_equal(F, F.T))
+    knobs = bool(args.wpr or args.pk or args.rpc or args.place)
+    # concurrent updates: their own kernel where the library takes it, else
+    # the table kernels, whose shape is reported
+    concurrent = (args.mode == "cupim" and infl == P.PDIT_INFLUENCE_AUTO and n <= 128 and symmetric and plain
+                  and top <= 127 and not knobs)
+    if args.mode == "cupim" and infl == P.PDIT_INFLUENCE_AUTO and not concurrent:
+        infl = P.PDIT_INFLUENCE_TABLE
     P.pdit_set_influence(q, infl)
     pt = args.mode == "pt"
     ladder = 10
@@ -827,7 +878,8 @@ def main():
     # roofline of the sweep kernel: shared-memory bound
     props = torch.cuda.get_device_properties(dev)
     dt_bytes = 1 if max(abs(int(D.max())), abs(int(F.max()))) <= 127 else 2
-    general = not (np.array_equal(D, D.T) and np.array_equal(F, F.T))
+    general = not symmetric
+    form = mm_form(n, top, general, plain)
     bpu = method_bytes_per_update(n, accept_frac, general)
     bpu_design = algorithmic_bytes_per_update(n, dt_bytes, accept_frac, shape["pending_swaps"], general)
     basis = (("16 N + A (8 N^2 + 16 N): the method's traffic with a rank-2 table rewrite per accepted swap "
@@ -845,6 +897,22 @@ def main():
         basis = ("(17 + dt) N + A (2 N dt + 8 N): the flow-class kernel's gathers plus, per accepted "
                  "swap, at most two D rows and the G vector (A counts swaps within a class too)")
         kname = "class_kernel<int8,%d,%d>" % (shape["candidates_per_thread"], shape["warps_per_replica"])
+    elif concurrent:
+        kname = "concurrent_kernel<%d>" % -(-n // 16)
+        # no table and no gathers: the method's figure does not apply
+        bpu = bpu_design = None
+        basis = "none: one product of depth 2N per iteration (pdit_concurrent.cu)"
+        macs = 2 * (16 * -(-n // 16)) ** 2
+        alu = {"op": "mma.sync f16 multiply-add", "per_update": macs, "achieved_ops_per_s": macs * upd_rank / kernel_s,
+               "peak_key": "mma_f16_macs_per_clk_sm"}
+    elif products and form is not None and not args.wpr:
+        # no table: the kernel's own traffic is the figure
+        bpu = bpu_design = mm_bytes_per_update(n, accept_frac, form)
+        basis = "the tensor-core product kernel's own shared-memory traffic (mm_bytes_per_update, %s form)" % form
+        kname = "mm_kernel<%d,%d,%s>" % (shape["candidates_per_thread"], mm_shape(n)[1], form)
+        macs = mm_macs_per_update(n, form)
+        alu = {"op": "mma.sync f16 multiply-add", "per_update": macs, "achieved_ops_per_s": macs * upd_rank / kernel_s,
+               "peak_key": "mma_f16_macs_per_clk_sm"}
     elif products:
         # no table: the kernel's own traffic is the design figure; the
         # method's figure stays the basis of `achieved`
@@ -852,8 +920,14 @@ def main():
         parts = dot_parts(replicas, shape["ctas"] * shape["replicas_per_cta"], 4 if pt else sweeps, pt)
         kname = dot_kernel_name(shape["candidates_per_thread"], shape["warps_per_replica"], n, parts)
         dp4a = product_dp4a_per_update(n)
-        alu = {"op": "dp4a", "per_update": dp4a, "achieved_ops_per_s": dp4a * upd_rank / kernel_s}
-    achieved = bpu * upd_rank / kernel_s / 1e9
+        alu = {"op": "dp4a", "per_update": dp4a, "achieved_ops_per_s": dp4a * upd_rank / kernel_s,
+               "peak_key": "dp4a_ops_per_clk_sm"}
+    elif not general and n <= 32 and shape["pending_swaps"] == 1 and shape["warps_per_replica"] == 1 and \
+            args.mode != "cupim":
+        # the table's row in registers and a copy in shared memory: the
+        # method's traffic, of which the kernel moves a part
+        kname = "small_kernel<%d>" % (16 if n <= 16 else 24 if n <= 24 else 32)
+    achieved = bpu * upd_rank / kernel_s / 1e9 if bpu is not None else None
     sm_mhz = clk.get("sm_mhz") or 0.0
     sms = props.multi_processor_count
     if peaks and sm_mhz:
@@ -861,10 +935,10 @@ def main():
         peak_source = ("measured: pdit_probe_peaks %.1f B/clk/SM (conflict-free 128-bit ld.shared) x %d SMs x "
                        "median SM clock under load (%s MHz)" % (peaks["smem_bytes_per_clk_sm"], sms, sm_mhz))
         if alu is not None:
-            alu["peak_ops_per_s"] = sms * peaks["dp4a_ops_per_clk_sm"] * sm_mhz * 1e6
+            per_clk = peaks[alu["peak_key"]]
+            alu["peak_ops_per_s"] = sms * per_clk * sm_mhz * 1e6
             alu["frac"] = alu["achieved_ops_per_s"] / alu["peak_ops_per_s"]
-            alu["peak_source"] = "measured: pdit_probe_peaks %.1f dp4a/clk/SM x %d SMs x %s MHz" % (
-                peaks["dp4a_ops_per_clk_sm"], sms, sm_mhz)
+            alu["peak_source"] = "measured: pdit_probe_peaks %.1f /clk/SM x %d SMs x %s MHz" % (per_clk, sms, sm_mhz)
     else:
         peak = sms * SMEM_BYTES_PER_CLK * sm_mhz * 1e6 / 1e9 if sm_mhz else None
         peak_source = "derived: %d SMs x %d B/clk x median SM clock under load (%s MHz)" % (
@@ -889,7 +963,8 @@ def main():
                                              WORKLOAD_TEXT[args.workload])
                    if args.workload in WORKLOAD_TEXT else args.workload,
                    "mode": args.mode,
-                   "update": "flow classes" if class_path else ("dot products" if products else "table"),
+                   "update": "flow classes" if class_path else ("concurrent products" if concurrent
+                                                                     else "products" if products else "table"),
                    "replicas_per_gpu": replicas, "sweeps": sweeps, "schedule": "pt ladder" if pt else kind, "seed": 0,
                    "global_batch": replicas * world, "seq_len": n,
                    "parallelism": "replicas sharded over %d GPU(s)" % world,
@@ -908,12 +983,13 @@ def main():
         "clocks": {"sm_mhz": clk.get("sm_mhz"), "sm_max_mhz": clk.get("sm_max_mhz"),
                    "reasons": clk.get("reasons"), "samples": clk.get("samples")},
         "roofline": {"bound": "smem", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                     "frac": (achieved / peak) if peak else None, "traffic": traffic,
+                     "frac": (achieved / peak) if peak and achieved is not None else None, "traffic": traffic,
                      "kernel": kname,
                      "bytes_per_update": bpu,
                      "bytes_per_update_basis": basis,
                      "design_bytes_per_update": bpu_design,
-                     "design_frac": (bpu_design * upd_rank / kernel_s / 1e9 / peak) if peak else None,
+                     "design_frac": (bpu_design * upd_rank / kernel_s / 1e9 / peak) if peak and bpu_design is not None
+                     else None,
                      "peak_source": peak_source, "alu": alu},
         "wall_s_timed_region": wall,
     }

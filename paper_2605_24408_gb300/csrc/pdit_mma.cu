@@ -40,14 +40,16 @@
 // 64 replicas, 1.6 (N = 33) to 6.6 (N = 112) with 4096.
 //
 // Bound: the latency of an update's chain of about 450 instructions a warp
-// (issue slots 50% busy, 16 warps an SM at the register limit; shared-memory
-// pipe 60%, tensor pipe 23%). Byte permutes that form a gather's address from
+// (issue slots 45% busy, 15 warps an SM at the register limit; shared-memory
+// pipe 67%, tensor pipe 26%). Byte permutes that form a gather's address from
 // its row's, warp-uniform control and replicas paired in warps from the first
 // took N = 100, 4096 replicas, from 2.13e9 to 2.39e9 updates/s (1.12e9 with
 // the dot-product kernel); N = 256, 2048 replicas: 7.3e8 (1.6e8 with the table
 // kernels). Bytes instead of f16 words for the vectors, with h in registers,
 // cut the wavefronts by a fifth but were slower (2.03e9: more instructions);
-// products formed one location ahead by warps of their own were too (1.78e9).
+// products formed one location ahead by warps of their own were too (1.78e9);
+// two accumulators a tile, the scaled row's load ahead of the gathers and a
+// total by butterfly changed nothing.
 #include <type_traits>
 
 #include "pdit_f16.cuh"
