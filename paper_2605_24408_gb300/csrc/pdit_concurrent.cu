@@ -26,10 +26,11 @@
 // energies are exact, so the trajectories equal the table kernels'.
 //
 // Bound: an iteration's latency, about 17000 clocks at N = 100, 7000 of them
-// the product (two warps a scheduler reach half of mma.sync's rate; loads of a
-// step ahead of its products made no difference) and 2000 to 4000 the
+// the two products (two warps a scheduler reach half of mma.sync's rate; loads
+// of a step ahead of its products made no difference) and 2000 to 4000 the
 // matching, two CTAs an SM overlapped. N = 100, 4096 replicas x 60 iterations:
-// 7.8 ms (21.6 ms with the table kernels, which update every table entry for
+// 7.0 ms (7.8 ms with both products at this size too, 8.8 ms with two warps a
+// row tile; 21.6 ms with the table kernels, which update every table entry for
 // every accepted swap); N = 12, 64 replicas: 0.21 ms (0.57 ms).
 #include "pdit_f16.cuh"
 #include "pdit_sweep.cuh"
@@ -42,9 +43,16 @@ struct CcShape {
     static constexpr int GS = 16 * (MT | 1);  // row stride of D and G, bytes
     static constexpr int FS = 256;            // of F: an entry's address is its row's with the column for the low byte
     static constexpr int CTAS = (MT >= 7 ? 512 : MT >= 5 ? 640 : 768) / T;  // resident CTAs an SM aimed at (more spill)
+    // S = J + J^T, J = D G exchanged through shared memory, where that takes
+    // no CTA away; else both products. 4096 replicas x 60 iterations, J or
+    // both: N = 100 7.0 or 7.8 ms; N = 96 5.8 or 5.2, N = 64 2.2 or 2.0 (J's
+    // memory leaves fewer CTAs an SM); N = 128: J leaves one.
+    static constexpr bool TR = MT == 7;
+    static constexpr int CS = NP + 4;  // row stride of J, floats: the transposed reads of a warp in distinct banks (NP = 112)
     // shared memory, bytes (F first: its rows are 256-byte aligned)
     static constexpr int oF = 0, oD = oF + NP * FS, oG = oD + NP * GS, oP = oG + NP * GS, oS = oP + 128,
-                         oB = oS + 4 * (NP + 8), oTk = oB + 2 * 4 * 128, oX = oTk + 128, bytes = oX + 32;
+                         oB = oS + 4 * (NP + 8), oTk = oB + 2 * 4 * 128, oX = oTk + 128,
+                         oJ = oX + 32, bytes = oJ + (TR ? 4 * NP * CS : 0);
     __host__ __device__ static constexpr int slot(int x) {
         return 8 * ((x % LC) >> 1) + 2 * (x / LC) + (x & 1);
     }
@@ -134,7 +142,8 @@ __device__ __forceinline__ void cc_energies(unsigned char *sm, int n, float (&ac
             const uint32_t x = *reinterpret_cast<const uint32_t *>(bG + 8 * t * GS + 16 * s);
             const uint32_t y = *reinterpret_cast<const uint32_t *>(bD + 8 * t * GS + 16 * s);
             mma_f16(acc[t], aD, make_uint2(__byte_perm(x, 0, 0x4140), __byte_perm(x, 0, 0x4342)));
-            mma_f16(acc[t], aG, make_uint2(__byte_perm(y, 0, 0x4140), __byte_perm(y, 0, 0x4342)));
+            if constexpr (!S::TR)
+                mma_f16(acc[t], aG, make_uint2(__byte_perm(y, 0, 0x4140), __byte_perm(y, 0, 0x4342)));
         }
     }
     // diagonal: rows 16 m + g and 16 m + 8 + g are columns 2 q + e = g of tiles 2 m, 2 m + 1
@@ -146,6 +155,16 @@ __device__ __forceinline__ void cc_energies(unsigned char *sm, int n, float (&ac
             d0 = g & 1 ? acc[2 * t][1] : acc[2 * t][0];
             d1 = g & 1 ? acc[2 * t + 1][3] : acc[2 * t + 1][2];
         }
+    float *J = reinterpret_cast<float *>(sm + S::oJ) + (16 * m + g) * S::CS;
+    if constexpr (S::TR) {
+#pragma unroll
+        for (int t = 0; t < NT; ++t) {
+            *reinterpret_cast<float2 *>(J + 8 * t + 2 * q) = make_float2(acc[t][0], acc[t][1]);
+            *reinterpret_cast<float2 *>(J + 8 * S::CS + 8 * t + 2 * q) = make_float2(acc[t][2], acc[t][3]);
+        }
+        d0 += d0;
+        d1 += d1;
+    }
     const int x0 = LC * (g >> 1) + 4 * m + (g & 1), x1 = x0 + 2;  // locations of this lane's rows
     if (q == g >> 1) {
         // a location beyond n: energies of +infinity, weights of 0
@@ -153,6 +172,16 @@ __device__ __forceinline__ void cc_energies(unsigned char *sm, int n, float (&ac
         diag[S::diag(x1)] = x1 < n ? d1 : __int_as_float(0xFF800000);
     }
     __syncthreads();
+    if constexpr (S::TR) {
+        const float *Jt = reinterpret_cast<const float *>(sm + S::oJ) + 2 * q * S::CS + 16 * m + g;
+#pragma unroll
+        for (int t = 0; t < NT; ++t) {
+            acc[t][0] += Jt[8 * t * S::CS];
+            acc[t][1] += Jt[(8 * t + 1) * S::CS];
+            acc[t][2] += Jt[8 * t * S::CS + 8];
+            acc[t][3] += Jt[(8 * t + 1) * S::CS + 8];
+        }
+    }
     const float s0 = diag[S::diag(x0)], s1 = diag[S::diag(x1)];
     const float *dq = diag + (LC + 2) * q;
     const unsigned char *rD = sm + S::oD + (16 * m + g) * GS + LC * q, *rG = rD + (S::oG - S::oD);
