@@ -901,8 +901,8 @@ def main():
         kname = "concurrent_kernel<%d>" % -(-n // 16)
         # no table and no gathers: the method's figure does not apply
         bpu = bpu_design = None
-        basis = "none: one product of depth 2N per iteration (pdit_concurrent.cu)"
-        macs = 2 * (16 * -(-n // 16)) ** 2
+        basis = "none: products of the permuted flow, once per iteration (pdit_concurrent.cu)"
+        macs = (1 if -(-n // 16) == 7 else 2) * (16 * -(-n // 16)) ** 2
         alu = {"op": "mma.sync f16 multiply-add", "per_update": macs, "achieved_ops_per_s": macs * upd_rank / kernel_s,
                "peak_key": "mma_f16_macs_per_clk_sm"}
     elif products and form is not None and not args.wpr:
