@@ -283,7 +283,8 @@ typedef struct pdit_opts {
     uint32_t instance_id;   /* Philox counter word 0; default 0 */
     uint32_t replica_base;  /* global id of this call's replica 0 (counter word 1); default 0 */
     int mode;               /* PDIT_MODE_ANNEAL (default), _PT, _FIXED or _CUPIM (one iteration per sweep) */
-    const float *beta;      /* anneal: [sweeps]; PT: [ladder_len], rung 0 = smallest beta; fixed: [replicas] */
+    const float *beta;      /* anneal: [sweeps]; PT: [ladder_len], rung 0 = smallest beta; fixed: [replicas].
+                               Finite and >= 0; under an infinite beta or a NaN every location stays */
     int ladder_len;         /* PT: replicas per set (2..64); replicas % ladder_len == 0 */
     int exchange_period;    /* PT: sweeps between exchanges (paper: 4) */
     int timeout_periods;    /* PT: periods without a top-rung swap before top<->bottom (paper: 100); 0 = off */

@@ -314,7 +314,8 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
-// The draw by 64-bit integer prefix sums. Ends with the group synchronised.
+// The draw by 64-bit integer prefix sums; the low byte of `tag` is the
+// location that draws. Ends with the group synchronised.
 template <int MAXK, int WPR, typename Fac>
 __device__ __forceinline__ int3 eq5_draw_exact(const int (&dc)[MAXK], Fac fac, int n, int t, float beta,
                                                unsigned long long draw, int tag, int bar, GroupScratch *gs) {
@@ -365,7 +366,9 @@ __device__ __forceinline__ int3 eq5_draw_exact(const int (&dc)[MAXK], Fac fac, i
     const unsigned long long excl = incl - lsum;
     const unsigned long long tdraw = __umul64hi(draw, total);
     const bool own = (tdraw >= excl) && (tdraw < incl);
-    int jloc = 0, dsel = 0, fsel = 0;
+    // no outcome has a weight (beta infinite or not a number), so no thread
+    // owns the draw: the location stays
+    int jloc = tag & 0xFF, dsel = 0, fsel = 0;
     if (own) {
         int kk = MAXK - 1;
 #pragma unroll
@@ -380,14 +383,15 @@ __device__ __forceinline__ int3 eq5_draw_exact(const int (&dc)[MAXK], Fac fac, i
     int js, dstar, fb;
     if constexpr (WPR > 1) {
         // both below 2^8 (n <= 256)
-        if (own) *reinterpret_cast<int2 *>(&gs->sel_jf) = make_int2(jloc | (fsel << 8) | (tag << 16), dsel);
+        if (own || (total == 0ull && t == 0))
+            *reinterpret_cast<int2 *>(&gs->sel_jf) = make_int2(jloc | (fsel << 8) | (tag << 16), dsel);
         group_sync<WPR>(bar);
         const int2 sel = *reinterpret_cast<const int2 *>(&gs->sel_jf);
         js = sel.x & 0xFF;
         fb = (sel.x >> 8) & 0xFF;
         dstar = sel.y;
     } else {
-        const int src = __ffs(__ballot_sync(kFull, own)) - 1;
+        const int src = (__ffs(__ballot_sync(kFull, own)) - 1) & 31;  // (no owner: any lane's)
         js = __shfl_sync(kFull, jloc, src);
         dstar = __shfl_sync(kFull, dsel, src);
         fb = __shfl_sync(kFull, fsel, src);
