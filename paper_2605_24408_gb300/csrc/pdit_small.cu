@@ -180,6 +180,7 @@ __device__ __forceinline__ void run_small_replica(const SweepArgs &a, int r, int
             float incl = w, total = w;
 #pragma unroll
             for (int q = 0; q < NP / 4; ++q) add_scaled4(T[q], pu, reinterpret_cast<const V4 *>(sv)[q]);
+            __syncwarp();  // the reads of the table for this update's energies are done
             store();
 #pragma unroll
             for (int o = 1; o < (NP > 16 ? 32 : 16); o <<= 1) {

@@ -395,6 +395,7 @@ __device__ __forceinline__ int3 eq5_draw_exact(const int (&dc)[MAXK], Fac fac, i
         js = __shfl_sync(kFull, jloc, src);
         dstar = __shfl_sync(kFull, dsel, src);
         fb = __shfl_sync(kFull, fsel, src);
+        __syncwarp();  // (shuffles order no memory accesses)
     }
     return make_int3(js, dstar, fb);
 }
