@@ -492,12 +492,45 @@ bool use_cc_path(const pdit_qap *h, const pdit_opts *o) {
            h->force_place == PDIT_PLACE_AUTO && h->force_infl == PDIT_INFLUENCE_AUTO;
 }
 
+// Few replicas. The tensor-core product kernel's update is one chain however
+// few of its slots are in use; with few replicas an SM the kernels that put
+// several warps on a replica are faster: the dot-product kernel for
+// symmetric instances. The most replicas an SM at which `alt`, that kernel's
+// shape, is taken, from both kernels' times at 1 to 5 replicas an SM and 30
+// sizes of 105 to 256 locations. us an update, product kernel against dot
+// products: N = 120 1.04 / 1.01 at 1, 1.09 / 1.13 at 3; N = 160 1.27 / 1.03
+// at 1, 1.32 / 1.35 at 3; N = 176 1.52 / 1.36 at 3, 1.56 / 1.57 at 4; N = 200
+// 1.82 / 1.13 at 1, 1.91 / 1.90 at 4; N = 224 1.87 / 1.54 at 2, 1.90 / 2.46
+// at 3; N = 240 1.58 / 1.15 at 1, 1.62 / 1.63 at 2. Tempering gains less: a
+// launch of few sweeps also loads and stores the permuted matrices (N = 176
+// 0.83 of the product kernel's time at 1, 1.07 at 3).
+int few_replicas(const pdit_qap *h, const Plan &alt, bool pt) {
+    const int n = h->n;
+    switch (alt.wpr) {
+    case 2: return !pt && n <= 128 ? 2 : 0;
+    case 4: return pt ? (n <= 192 ? 1 : 2) : (n <= 160 ? 2 : 3);
+    case 8: return n <= 224 ? 2 : 1;
+    default: return 0;
+    }
+}
+
+// The shape of a call with few replicas, where another kernel than the
+// tensor-core product kernel takes it; false where none does.
+bool few_plan(const pdit_qap *h, int replicas, bool pt, Plan *p, size_t reserve) {
+    const int per_sm = (replicas + h->num_sms - 1) / h->num_sms;
+    if (per_sm > 3 || mm_form(h) != pdit::kMmSymmetric) return false;
+    if (make_dot_plan(h, replicas, 0, p, reserve) == PDIT_OK && per_sm <= few_replicas(h, *p, pt)) return true;
+    *p = Plan();
+    return false;
+}
+
 // The product kernel of a call: tensor-core products where the instance
-// allows them and no wider mapping than a warp per replica is asked for, else
-// the dot-product kernel. `any`: also where the automatic rule prefers the
-// table kernels.
-int product_plan(const pdit_qap *h, int replicas, Plan *p, size_t reserve, bool any) {
+// allows them, no wider mapping than a warp per replica is asked for and the
+// replicas are not few, else the dot-product kernel. `any`: also where the
+// automatic rule prefers the table kernels.
+int product_plan(const pdit_qap *h, int replicas, bool pt, Plan *p, size_t reserve, bool any) {
     if (mm_eligible(h) && h->force_wpr <= 1) {
+        if (h->force_wpr == 0 && few_plan(h, replicas, pt, p, reserve)) return PDIT_OK;
         const int rc = make_mm_plan(h, replicas, p, reserve);
         if (rc != PDIT_ENOTSUP) return rc;
         *p = Plan();
@@ -531,10 +564,10 @@ int plan_for(const pdit_qap *h, const pdit_opts *o, Plan *p) {
     }
     if (h->force_infl == PDIT_INFLUENCE_PRODUCTS) {
         if (!dot_eligible(h) || o->mode == PDIT_MODE_CUPIM || o->tables) return PDIT_ENOTSUP;
-        return product_plan(h, o->replicas, p, 0, true);
+        return product_plan(h, o->replicas, o->mode == PDIT_MODE_PT, p, 0, true);
     }
     if (use_dot_path(h, o)) {
-        const int rc = product_plan(h, o->replicas, p, 0, false);
+        const int rc = product_plan(h, o->replicas, o->mode == PDIT_MODE_PT, p, 0, false);
         if (rc != PDIT_ENOTSUP) return rc;
         *p = Plan();  // no suitable dot shape: the table kernels
     }
@@ -549,12 +582,12 @@ int batch_plan(const pdit_qap *h, Plan *p, size_t reserve) {
     if (!h->cls || !h->use_cls) {
         if (h->force_infl == PDIT_INFLUENCE_PRODUCTS) {
             if (!dot_eligible(h)) return PDIT_ENOTSUP;
-            return product_plan(h, 1 << 28, p, reserve, true);
+            return product_plan(h, 1 << 28, false, p, reserve, true);
         }
         pdit_opts o;
         pdit_opts_init(&o);
         if (use_dot_path(h, &o)) {
-            const int rc = product_plan(h, 1 << 28, p, reserve, false);
+            const int rc = product_plan(h, 1 << 28, false, p, reserve, false);
             if (rc != PDIT_ENOTSUP) return rc;
             *p = Plan();
         }
@@ -1262,7 +1295,7 @@ int pdit_autotune(pdit_qap *h, int replicas, const float *beta, int sweeps, int 
     auto plan_ok = [&](const Knobs &k, Plan *p) {
         set(k);
         if (cls) return make_class_plan(h, replicas, k.wpr, p) == PDIT_OK;
-        if (k.infl == PDIT_INFLUENCE_PRODUCTS) return product_plan(h, replicas, p, 0, true) == PDIT_OK;
+        if (k.infl == PDIT_INFLUENCE_PRODUCTS) return product_plan(h, replicas, false, p, 0, true) == PDIT_OK;
         return make_plan(h, replicas, k.wpr, k.pk, p) == PDIT_OK;
     };
     // Candidates: the table placement (a caller's choice, else the built-in

@@ -1,0 +1,75 @@
+"""Calls with few replicas an SM, where the automatic choice takes a kernel
+that puts several warps on a replica instead of the tensor-core product
+kernel: which one runs on each side of the lines, and that replicas equal the
+CPU oracle's there; and the product kernel at those sizes when one warp per
+replica is asked for."""
+
+import numpy as np
+import pytest
+
+import oracle as O
+from gpu_common import check, device, host, library, sms
+from paper_2605_24408_gb300 import instances as G
+
+pytestmark = pytest.mark.gpu
+
+
+def compare(p, q, D, F, beta, S, R, mode="anneal", L=4):
+    kw, okw, step = {}, {}, 1
+    if mode == "pt":
+        kw = dict(mode=p.PDIT_MODE_PT, ladder_len=L, exchange_period=2, timeout_periods=2)
+        okw, step = dict(mode="pt", ladder_len=L, period=2, timeout=2), L
+    g = host(p.anneal_device(q, R, device(beta), S, 6, per_replica=True, **kw))
+    for lo in {0, (R - 1) // step * step - step * (3 if step == 1 else 0)}:
+        lo = max(0, lo)
+        hi = min(R, lo + 4)
+        r = O.anneal(D, F, beta, S, 6, lo, hi, threads=4, **okw)
+        check(g, r, slice(lo, hi))
+
+
+@pytest.mark.parametrize("n,per_sm,warps", [(112, 1, 1), (113, 2, 2), (128, 2, 2), (128, 3, 1), (129, 1, 1), (160, 2, 4),
+                                            (160, 3, 1), (161, 3, 4), (200, 3, 4), (200, 4, 1), (224, 2, 8), (224, 3, 1),
+                                            (225, 1, 8), (225, 2, 1), (256, 1, 8)])
+def test_symmetric(n, per_sm, warps):
+    """`warps` at per_sm replicas an SM: 1 is the product kernel (the first
+    call that fills the SM to per_sm), more the dot-product kernel (the last)."""
+    p = library()
+    D, F = G.dense_instance(n, seed=n)
+    S = 3
+    beta = O.beta_schedule("linear", S, O.beta_max(D, F))
+    R = sms() * per_sm if warps > 1 else sms() * (per_sm - 1) + 1
+    for infl in (p.PDIT_INFLUENCE_AUTO, p.PDIT_INFLUENCE_PRODUCTS):
+        with p.Qap(D, F) as q:
+            p.pdit_set_influence(q, infl)
+            shape = p.pdit_launch_shape(q, R)
+            assert shape["influence"] == "products" and shape["warps_per_replica"] == warps
+            compare(p, q, D, F, beta, S, R)
+
+
+@pytest.mark.parametrize("n,per_sm,dot", [(120, 1, False), (176, 1, True), (176, 2, False), (200, 2, True),
+                                          (200, 3, False), (224, 2, True), (240, 1, True), (240, 2, False)])
+def test_symmetric_tempering(n, per_sm, dot):
+    p = library()
+    D, F = G.dense_instance(n, seed=n + 1)
+    L, S = 4, 5
+    beta = O.beta_schedule("geometric", L, O.beta_max(D, F))
+    R = (sms() * per_sm if dot else sms() * (per_sm - 1) + L) // L * L
+    with p.Qap(D, F) as q:
+        # the dot-product kernel's permuted matrices are kept between exchange periods
+        o = p.opts(replicas=R, sweeps=S, mode=p.PDIT_MODE_PT, ladder_len=L)
+        assert (p.pdit_workspace_bytes(q, o) > R * n * n) == dot
+        compare(p, q, D, F, beta, S, R, "pt", L)
+
+
+@pytest.mark.parametrize("n", [113, 128, 129, 160, 161, 192, 193, 224, 225, 256])
+def test_product_kernel_with_one_warp_asked(n):
+    p = library()
+    D, F = G.dense_instance(n, seed=n)
+    S = 4
+    beta = O.beta_schedule("linear", S, O.beta_max(D, F))
+    with p.Qap(D, F) as q:
+        p.pdit_set_warps_per_replica(q, 1)
+        # (its shared memory does not depend on the replicas)
+        a, b = p.pdit_launch_shape(q, 1), p.pdit_launch_shape(q, 1 << 16)
+        assert a["influence"] == "products" and a["smem_bytes"] == b["smem_bytes"]
+        compare(p, q, D, F, beta, S, 5)
