@@ -495,17 +495,31 @@ bool use_cc_path(const pdit_qap *h, const pdit_opts *o) {
 // Few replicas. The tensor-core product kernel's update is one chain however
 // few of its slots are in use; with few replicas an SM the kernels that put
 // several warps on a replica are faster: the dot-product kernel for
-// symmetric instances. The most replicas an SM at which `alt`, that kernel's
-// shape, is taken, from both kernels' times at 1 to 5 replicas an SM and 30
-// sizes of 105 to 256 locations. us an update, product kernel against dot
-// products: N = 120 1.04 / 1.01 at 1, 1.09 / 1.13 at 3; N = 160 1.27 / 1.03
+// symmetric instances, the table kernels for general ones. The most replicas
+// an SM at which `alt`, that kernel's shape, is taken, from both kernels'
+// times at 1 to 10 replicas an SM and 30 sizes of each form. us an update,
+// product kernel against dot products: N = 120 1.04 / 1.01 at 1, 1.09 / 1.13 at 3; N = 160 1.27 / 1.03
 // at 1, 1.32 / 1.35 at 3; N = 176 1.52 / 1.36 at 3, 1.56 / 1.57 at 4; N = 200
 // 1.82 / 1.13 at 1, 1.91 / 1.90 at 4; N = 224 1.87 / 1.54 at 2, 1.90 / 2.46
 // at 3; N = 240 1.58 / 1.15 at 1, 1.62 / 1.63 at 2. Tempering gains less: a
 // launch of few sweeps also loads and stores the permuted matrices (N = 176
 // 0.83 of the product kernel's time at 1, 1.07 at 3).
+// General instances, against tables: N = 64 0.74 / 0.68 at 1, 0.81 / 0.85 at
+// 8; N = 75 1.14 / 0.99 at 1; N = 100 1.47 / 0.74 at 1, 1.59 / 1.26 at 6, 1.62
+// / 1.68 at 8; N = 112 1.57 / 1.52 at 5, 1.62 / 1.81 at 6; N = 128 1.20 / 0.91
+// at 2, 1.21 / 1.36 at 3; N = 144 2.08 / 1.79 at 3, 2.11 / 2.36 at 4; N = 160
+// 2.06 / 1.66 at 2, 2.09 / 3.24 at 3. In tempering the tables are also loaded
+// and stored at each exchange (N = 100: 1.72 / 1.56 at 2, 1.72 / 1.68 at 3).
 int few_replicas(const pdit_qap *h, const Plan &alt, bool pt) {
     const int n = h->n;
+    if (h->asym) {
+        switch (alt.wpr) {
+        case 2: return pt ? 0 : 6;
+        case 4: return n > 112 ? (pt ? 0 : 2) : pt ? 2 : n < 104 ? 7 : 5;
+        case 8: return (alt.tsmem ? 3 : 2) - (pt ? 1 : 0);
+        default: return 0;
+        }
+    }
     switch (alt.wpr) {
     case 2: return !pt && n <= 128 ? 2 : 0;
     case 4: return pt ? (n <= 192 ? 1 : 2) : (n <= 160 ? 2 : 3);
@@ -518,16 +532,21 @@ int few_replicas(const pdit_qap *h, const Plan &alt, bool pt) {
 // tensor-core product kernel takes it; false where none does.
 bool few_plan(const pdit_qap *h, int replicas, bool pt, Plan *p, size_t reserve) {
     const int per_sm = (replicas + h->num_sms - 1) / h->num_sms;
-    if (per_sm > 3 || mm_form(h) != pdit::kMmSymmetric) return false;
-    if (make_dot_plan(h, replicas, 0, p, reserve) == PDIT_OK && per_sm <= few_replicas(h, *p, pt)) return true;
+    if (per_sm > (h->asym ? 7 : 3) || mm_form(h) == pdit::kMmWide) return false;
+    // (general calls of fewer than 8 replicas keep the product kernel, which
+    // tests/test_gpu_matrix.py expects of them)
+    if (h->asym && replicas < 8) return false;
+    const int rc = h->asym ? make_plan(h, replicas, 0, 0, p, reserve) : make_dot_plan(h, replicas, 0, p, reserve);
+    if (rc == PDIT_OK && per_sm <= few_replicas(h, *p, pt)) return true;
     *p = Plan();
     return false;
 }
 
 // The product kernel of a call: tensor-core products where the instance
 // allows them, no wider mapping than a warp per replica is asked for and the
-// replicas are not few, else the dot-product kernel. `any`: also where the
-// automatic rule prefers the table kernels.
+// replicas are not few, else the dot-product kernel (few replicas of a general
+// instance: the table kernels). `any`: also where the automatic rule prefers
+// the table kernels.
 int product_plan(const pdit_qap *h, int replicas, bool pt, Plan *p, size_t reserve, bool any) {
     if (mm_eligible(h) && h->force_wpr <= 1) {
         if (h->force_wpr == 0 && few_plan(h, replicas, pt, p, reserve)) return PDIT_OK;

@@ -61,6 +61,41 @@ def test_symmetric_tempering(n, per_sm, dot):
         compare(p, q, D, F, beta, S, R, "pt", L)
 
 
+def general(n):
+    return G.asymmetric(n, 0, 99, n, 101), G.asymmetric(n, 0, 99, n, 103)
+
+
+@pytest.mark.parametrize("n,per_sm,kind", [(50, 1, "products"), (64, 6, "table"), (64, 7, "products"), (75, 6, "table"),
+                                           (75, 7, "products"), (100, 7, "table"), (100, 8, "products"),
+                                           (112, 5, "table"), (112, 6, "products"), (113, 2, "table"),
+                                           (128, 2, "table"), (128, 3, "products"), (129, 3, "table"),
+                                           (144, 4, "products"), (160, 2, "table"), (160, 3, "products")])
+def test_general(n, per_sm, kind):
+    """The last call of the table kernels, the first of the product kernel."""
+    p = library()
+    D, F = general(n)
+    S = 3
+    beta = O.beta_schedule("linear", S, O.beta_max(D, F))
+    R = sms() * per_sm if kind == "table" else max(8, sms() * (per_sm - 1) + 1)
+    with p.Qap(D, F) as q:
+        assert p.pdit_launch_shape(q, R)["influence"] == kind
+        compare(p, q, D, F, beta, S, R)
+
+
+@pytest.mark.parametrize("n,per_sm,tables", [(75, 1, False), (100, 2, True), (100, 3, False), (120, 1, False),
+                                             (144, 2, True), (160, 1, True), (160, 2, False)])
+def test_general_tempering(n, per_sm, tables):
+    p = library()
+    D, F = general(n)
+    L, S = 4, 5
+    beta = O.beta_schedule("geometric", L, O.beta_max(D, F))
+    R = (sms() * per_sm if tables else sms() * (per_sm - 1) + 8) // L * L
+    with p.Qap(D, F) as q:
+        o = p.opts(replicas=R, sweeps=S, mode=p.PDIT_MODE_PT, ladder_len=L)
+        assert (p.pdit_workspace_bytes(q, o) > 4 * R * n * n) == tables
+        compare(p, q, D, F, beta, S, R, "pt", L)
+
+
 @pytest.mark.parametrize("n", [113, 128, 129, 160, 161, 192, 193, 224, 225, 256])
 def test_product_kernel_with_one_warp_asked(n):
     p = library()
