@@ -157,6 +157,7 @@ __device__ __forceinline__ void run_class_replica(const SweepArgs &a, int r, int
             if (stop_now) break;
         }
         const float beta = (a.mode == 1 || a.mode == 2) ? beta_fixed : a.beta[s];
+        if (!sweep_moves(beta)) continue;
         for (int i0 = 0; i0 < n; i0 += 32) {
             const uint4 rw = philox4x32_10(a.inst, grep, (uint32_t)s, (uint32_t)(i0 + lane), a.key0, a.key1);
             const int cnt = min(32, n - i0);

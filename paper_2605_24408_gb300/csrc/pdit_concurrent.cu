@@ -68,11 +68,10 @@ struct CcRow {
     float v[LC];
 };
 
-// The exact draw (eq5_draw_exact) of location i for the four lanes of each
-// row; q: the lane's place, v: its outcomes LC q + k. Returns the outcome.
+// The exact draw (eq5_draw_exact) for the four lanes of each row; q: the
+// lane's place, v: its outcomes LC q + k. Returns the outcome.
 template <int LC>
-__device__ __noinline__ int cc_exact_draw(const CcRow<LC> d, int n, int i, int q, float beta,
-                                          unsigned long long draw) {
+__device__ __noinline__ int cc_exact_draw(const CcRow<LC> d, int n, int q, float beta, unsigned long long draw) {
     float dmin = __int_as_float(0x7F800000);
 #pragma unroll
     for (int k = 0; k < LC; ++k) dmin = fminf(dmin, d.v[k]);
@@ -101,8 +100,7 @@ __device__ __noinline__ int cc_exact_draw(const CcRow<LC> d, int n, int i, int q
             }
     }
     j = min(j, __shfl_xor_sync(kFull, j, 1));
-    j = min(j, __shfl_xor_sync(kFull, j, 2));
-    return j < n ? j : i;  // (no outcome has a weight: the location stays)
+    return min(j, __shfl_xor_sync(kFull, j, 2));
 }
 
 // G from the permutation, S and the swap energies (units of 2^-48) in `acc`.
@@ -283,9 +281,9 @@ __device__ __forceinline__ void cc_run_replica(const SweepArgs &a, int r, int pa
             if (*flag) break;
         }
         const float beta = a.beta[s];
-        // (never 0, so that an infinite energy always has weight 0; a beta
-        // that is not a number stays one, so that the exact draw decides)
-        const float kx = -beta * kLog2e * kCcScale, kb = kx > -1e-37f ? -1e-37f : kx;
+        if (!sweep_moves(beta)) continue;
+        // (never 0, so that an infinite energy always has weight 0)
+        const float kb = fminf(-beta * kLog2e * kCcScale, -1e-37f);
         // Philox(inst, replica, iteration, location): lanes 0, 2 of a row pair have half 0's, 1, 3 half 1's
         const uint4 rw = philox4x32_10(a.inst, grep, (uint32_t)s, (uint32_t)(row0 + 2 * (q & 1)), a.key0, a.key1);
         // ---- proposals: one row of the quad's two at a time; lane q keeps row q's (q < 2)
@@ -352,7 +350,7 @@ __device__ __forceinline__ void cc_run_replica(const SweepArgs &a, int r, int pa
 #pragma unroll
                 for (int k = 0; k < LC; ++k) row.v[k] = e[k / 2][2 * h + (k & 1)];
                 const uint32_t dlo = __shfl_sync(kFull, rw.x, h, 4);
-                const int jx = cc_exact_draw<LC>(row, n, i, q, beta, ((unsigned long long)dhi << 32) | dlo);
+                const int jx = cc_exact_draw<LC>(row, n, q, beta, ((unsigned long long)dhi << 32) | dlo);
                 float dx = 0.0f;
 #pragma unroll
                 for (int k = 0; k < LC; ++k)

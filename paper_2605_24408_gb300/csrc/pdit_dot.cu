@@ -194,6 +194,7 @@ __device__ __forceinline__ void run_dot_replica(const SweepArgs &a, int r, int t
             if (stop_now) break;
         }
         const float beta_now = (a.mode == 1 || a.mode == 2) ? beta_fixed : a.beta[s];
+        if (!sweep_moves(beta_now)) continue;
         // One p-dit update of location i with the influence entries rowv[k] =
         // I[i][p(j)], colv[k] = I[j][p(i)] of this thread's locations j. With
         // `fix`, rowB and colB hold the entries of the next location i + 1

@@ -145,9 +145,10 @@ __device__ __forceinline__ int mm_top(int) { return 0x7FFFFFFF; }
 __device__ __forceinline__ float mm_min(float a, float b) { return fminf(a, b); }
 __device__ __forceinline__ int mm_min(int a, int b) { return min(a, b); }
 
-// The exact draw (eq5_draw_exact) of location i for one replica's LPR threads.
+// The exact draw (eq5_draw_exact) for one replica's LPR threads; beyond n
+// where no outcome has a weight.
 template <int K, int LPR, typename V>
-__device__ __noinline__ int mm_exact_draw(const MmVals<K, V> d, int n, int i, int t, float scale, float beta,
+__device__ __noinline__ int mm_exact_draw(const MmVals<K, V> d, int n, int t, float scale, float beta,
                                           unsigned long long draw, unsigned mask) {
     V dmin = mm_top(V());
 #pragma unroll
@@ -177,7 +178,7 @@ __device__ __noinline__ int mm_exact_draw(const MmVals<K, V> d, int n, int i, in
         if (tdraw >= excl && excl + pre[k] > tdraw) j = t * K + k;
 #pragma unroll
     for (int o = LPR / 2; o; o >>= 1) j = min(j, __shfl_xor_sync(mask, j, o, LPR));
-    return j < n ? j : i;  // (no outcome has a weight: the location stays)
+    return j;
 }
 
 // Address of entry byte8(v, k) of the table row at `row`.
@@ -481,7 +482,7 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
         }
         // (never 0, so that an infinite energy always has weight 0; a beta
         // that is not a number stays one, so that the exact draw decides)
-        const float kx = -beta_of(s) * kLog2e * (WIDE ? 2.0f : kScale), kb = kx > -1e-37f ? -1e-37f : kx;
+        const float kb = min_nan(-beta_of(s) * kLog2e * (WIDE ? 2.0f : kScale), -1e-37f);
         uint32_t rhi = 0;  // high words of the draws of LPR locations
         int moves = 0;
         // location i = ti K + ki
@@ -629,8 +630,9 @@ __device__ __forceinline__ void mm_run_block(const SweepArgs &a, int r0, int par
                 int v = __shfl_sync(kFull, (t << 8) | kk | (int)(__byte_perm(p8.x, p8.y, kk) << 16), __ffs(ball) - 1);
                 if (__any_sync(kFull, ball == 0)) {
                     const uint32_t dlo = philox4x32_10(a.inst, grep, (uint32_t)s, (uint32_t)i, a.key0, a.key1).x;
-                    const int js = mm_exact_draw<K, LPR>(e, n, i, t, kScale, beta_of(s), ((unsigned long long)dhi << 32) | dlo, kFull);
+                    const int jx = mm_exact_draw<K, LPR>(e, n, t, kScale, beta_of(s), ((unsigned long long)dhi << 32) | dlo, kFull);
                     if (ball == 0) {
+                        const int js = jx < n ? jx : i;  // (no outcome has a weight: the location stays)
                         const int tx = js / K, kx = js - tx * K;
                         v = (tx << 8) | kx | (lds_u8(aP + 8 * tx + kx) << 16);
                     }

@@ -198,7 +198,8 @@ __device__ __forceinline__ void run_small_replica(const SweepArgs &a, int r, int
                 const int dc[1] = {(int)e.d};
                 const unsigned long long draw = ((unsigned long long)__shfl_sync(kFull, rw.y, i) << 32) |
                                                 (unsigned long long)__shfl_sync(kFull, rw.x, i);
-                js = eq5_draw_exact<1, 1>(dc, [&](int) { return p; }, n, lane, beta, draw, i, 0, nullptr).x;
+                js = eq5_draw_exact<1, 1>(dc, [&](int) { return p; }, n, lane, beta, draw, 0, 0, nullptr).x;
+                if (!sweep_moves(beta)) js = i;
             }
             pu = 0;
             if (js != i) {

@@ -314,8 +314,14 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
-// The draw by 64-bit integer prefix sums; the low byte of `tag` is the
-// location that draws. Ends with the group synchronised.
+// A sweep under a beta that is not finite moves nothing: every weight is 0.
+// The draws below need an outcome with a weight, so such sweeps are left out
+// (one compare a sweep; a test in the draw itself cost kernels of several
+// warps a replica up to 6%).
+__device__ __forceinline__ bool sweep_moves(float beta) { return fabsf(beta) <= 3.402823466e38f; }
+
+// The draw by 64-bit integer prefix sums; some outcome has a weight. Ends
+// with the group synchronised.
 template <int MAXK, int WPR, typename Fac>
 __device__ __forceinline__ int3 eq5_draw_exact(const int (&dc)[MAXK], Fac fac, int n, int t, float beta,
                                                unsigned long long draw, int tag, int bar, GroupScratch *gs) {
@@ -366,9 +372,7 @@ __device__ __forceinline__ int3 eq5_draw_exact(const int (&dc)[MAXK], Fac fac, i
     const unsigned long long excl = incl - lsum;
     const unsigned long long tdraw = __umul64hi(draw, total);
     const bool own = (tdraw >= excl) && (tdraw < incl);
-    // no outcome has a weight (beta infinite or not a number), so no thread
-    // owns the draw: the location stays
-    int jloc = tag & 0xFF, dsel = 0, fsel = 0;
+    int jloc = 0, dsel = 0, fsel = 0;
     if (own) {
         int kk = MAXK - 1;
 #pragma unroll
@@ -383,15 +387,14 @@ __device__ __forceinline__ int3 eq5_draw_exact(const int (&dc)[MAXK], Fac fac, i
     int js, dstar, fb;
     if constexpr (WPR > 1) {
         // both below 2^8 (n <= 256)
-        if (own || (total == 0ull && t == 0))
-            *reinterpret_cast<int2 *>(&gs->sel_jf) = make_int2(jloc | (fsel << 8) | (tag << 16), dsel);
+        if (own) *reinterpret_cast<int2 *>(&gs->sel_jf) = make_int2(jloc | (fsel << 8) | (tag << 16), dsel);
         group_sync<WPR>(bar);
         const int2 sel = *reinterpret_cast<const int2 *>(&gs->sel_jf);
         js = sel.x & 0xFF;
         fb = (sel.x >> 8) & 0xFF;
         dstar = sel.y;
     } else {
-        const int src = (__ffs(__ballot_sync(kFull, own)) - 1) & 31;  // (no owner: any lane's)
+        const int src = __ffs(__ballot_sync(kFull, own)) - 1;
         js = __shfl_sync(kFull, jloc, src);
         dstar = __shfl_sync(kFull, dsel, src);
         fb = __shfl_sync(kFull, fsel, src);
@@ -1047,6 +1050,7 @@ __device__ __forceinline__ void run_replica(const SweepArgs &a, int part_arg, in
             if (stop_now) break;
         }
         const float beta = (a.mode == 1 || a.mode == 2) ? beta_fixed : a.beta[s];
+        if (!sweep_moves(beta)) continue;
         if (a.mode == 3) {
             // ---- concurrent updates (one iteration): proposals drawn from a
             // snapshot of the swap energies, ranked by energy change (ties to
