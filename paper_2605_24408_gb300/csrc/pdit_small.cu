@@ -170,6 +170,7 @@ __device__ __forceinline__ void run_small_replica(const SweepArgs &a, int r, int
         const float ul = __uint2float_rn(rw.y >> 8) * 5.9604644775390625e-08f;
         int moves = 0;
         for (int i = 0; i < n; ++i) {
+            __syncwarp();  // the reads of the table for this update's energies are done
             const int nxt = i + 1 < n ? i + 1 : 0;
             const float u01 = __shfl_sync(kFull, ul, i);
             const int fnxt = __shfl_sync(kFull, p, nxt);
@@ -180,7 +181,6 @@ __device__ __forceinline__ void run_small_replica(const SweepArgs &a, int r, int
             float incl = w, total = w;
 #pragma unroll
             for (int q = 0; q < NP / 4; ++q) add_scaled4(T[q], pu, reinterpret_cast<const V4 *>(sv)[q]);
-            __syncwarp();  // the reads of the table for this update's energies are done
             store();
 #pragma unroll
             for (int o = 1; o < (NP > 16 ? 32 : 16); o <<= 1) {
