@@ -593,25 +593,50 @@ int plan_for(const pdit_qap *h, const pdit_opts *o, Plan *p) {
     return make_plan(h, o->replicas, h->force_wpr, h->force_pk, p, 0, o->mode == PDIT_MODE_CUPIM);
 }
 
-// Plan of one instance in a multi-instance launch (batches, the server):
-// the dot kernel where the automatic rule takes it, else the table kernels;
-// the kernels keep their descriptor in `reserve` bytes of static shared
-// memory.
-int batch_plan(const pdit_qap *h, Plan *p, size_t reserve) {
+// Whether a multi-instance launch of `load` replicas in all takes `alt`, the
+// shape of the kernel that an instance runs where the tensor-core product
+// kernel does not, instead of that kernel: where the launch is one round of
+// alt's resident replicas and alt puts several warps on a replica. Time of a
+// batch, alt / product kernel, inside the round and beyond it: general N = 80
+// 0.75 and 1.27, N = 100 0.71 and 1.15, N = 112 0.58 and 1.15, N = 128 0.73 and
+// 1.46, N = 160 0.81 and 1.60 (N = 76, two warps: 1.05); wide N = 120 0.87 and
+// 1.73, N = 128 0.91 and 1.79 (N = 112: 1.13); symmetric N = 212 0.88 and 1.74,
+// N = 224 0.91 and 1.80 (N = 225: 1.11; at 208 and below dot products: 1.01).
+bool few_load(const pdit_qap *h, const Plan &alt, long long load) {
+    if (alt.wpr < 4 || load > (long long)alt.grid * alt.groups) return false;
+    if (h->asym) return true;
+    return mm_form(h) == pdit::kMmWide ? h->n > 112 : !alt.dot && h->n <= 224;
+}
+
+// Plan of one instance in a multi-instance launch (batches, the server) of
+// `load` replicas in all: the product kernels where the automatic rule takes
+// them, else the table kernels; the kernels keep their descriptor in
+// `reserve` bytes of static shared memory.
+int batch_plan(const pdit_qap *h, long long load, Plan *p, size_t reserve) {
+    const int full = 1 << 28;  // as many replicas per CTA as fit
     if (!h->cls || !h->use_cls) {
         if (h->force_infl == PDIT_INFLUENCE_PRODUCTS) {
             if (!dot_eligible(h)) return PDIT_ENOTSUP;
-            return product_plan(h, 1 << 28, false, p, reserve, true);
+            return product_plan(h, full, false, p, reserve, true);
         }
         pdit_opts o;
         pdit_opts_init(&o);
         if (use_dot_path(h, &o)) {
-            const int rc = product_plan(h, 1 << 28, false, p, reserve, false);
+            if (mm_eligible(h) && h->force_wpr == 0) {
+                int rc = dot_eligible(h) ? auto_dot_plan(h, full, p, reserve) : PDIT_ENOTSUP;
+                if (rc == PDIT_ENOTSUP) {
+                    *p = Plan();
+                    rc = make_plan(h, full, 0, 0, p, reserve);
+                }
+                if (rc == PDIT_OK && few_load(h, *p, load)) return PDIT_OK;
+                *p = Plan();
+            }
+            const int rc = product_plan(h, full, false, p, reserve, false);
             if (rc != PDIT_ENOTSUP) return rc;
             *p = Plan();
         }
     }
-    return make_plan(h, 1 << 28, h->force_wpr, h->force_pk, p, reserve);
+    return make_plan(h, full, h->force_wpr, h->force_pk, p, reserve);
 }
 
 struct Workspace {
@@ -1870,10 +1895,12 @@ int pdit_batch_create(const pdit_batch_item *items, int count, uint32_t flags, p
     std::vector<Plan> plans((size_t)count);
     std::vector<size_t> ws_off((size_t)count);
     size_t ws_total = 0;
+    long long load = 0;  // replicas of the launch
+    for (int k = 0; k < count; ++k) load += items[k].replicas;
     for (int k = 0; k < count; ++k) {
         pdit_qap *h = items[k].qap;
         // the multi-instance kernels keep their instance descriptor in static shared memory
-        int rc = batch_plan(h, &plans[k], kBatchStaticSmem);
+        int rc = batch_plan(h, load, &plans[k], kBatchStaticSmem);
         if (rc) {
             delete b;
             return rc;
@@ -2152,10 +2179,12 @@ size_t request_footprint(const ServerRequest &r, const Plan &p) {
            1024;
 }
 
-int admit(pdit_server *s, ServerRequest *r) {
+// `load`: replicas of the requests that run or wait.
+int admit(pdit_server *s, ServerRequest *r, long long load) {
     int rc = qap_prepare(r->n, r->D.data(), r->F.data(), &r->qap);
     if (rc) return rc;
-    rc = batch_plan(r->qap, &r->plan, kBatchStaticSmem);
+    r->plan = Plan();  // (an earlier attempt that did not fit may have left one)
+    rc = batch_plan(r->qap, load, &r->plan, kBatchStaticSmem);
     if (rc) return rc;
     const size_t fp = request_footprint(*r, r->plan);
     // wait for memory; a request larger than the budget is admitted alone,
@@ -2385,9 +2414,12 @@ int pdit_server_tick(pdit_server *s, int *active, int *queued) {
     // 1. admit queued requests (FIFO) while slots and device memory allow
     {
         std::lock_guard<std::mutex> lock(s->mu);
+        long long load = 0;
+        for (const ServerRequest *r : s->active) load += r->replicas;
+        for (const ServerRequest *r : s->queue) load += r->replicas;
         while (!s->queue.empty() && (int)s->active.size() < s->max_active) {
             ServerRequest *r = s->queue.front();
-            const int rc = admit(s, r);
+            const int rc = admit(s, r, load);
             if (rc == 1) {  // does not fit yet: release what admit created, retry later
                 qap_destroy(r->qap);
                 r->qap = nullptr;

@@ -108,3 +108,61 @@ def test_product_kernel_with_one_warp_asked(n):
         a, b = p.pdit_launch_shape(q, 1), p.pdit_launch_shape(q, 1 << 16)
         assert a["influence"] == "products" and a["smem_bytes"] == b["smem_bytes"]
         compare(p, q, D, F, beta, S, 5)
+
+
+def instance(kind, n):
+    if kind == "general":
+        return general(n)
+    if kind == "wide":
+        return G.dense_symmetric(n, 0, 999, n, tag=23), G.dense_symmetric(n, 0, 999, n, tag=33)
+    return G.dense_instance(n, seed=n)
+
+
+MULTI = [("general", 76, False), ("general", 80, True), ("general", 100, True), ("general", 128, True),
+         ("general", 160, True), ("wide", 112, False), ("wide", 128, True), ("dense", 200, False), ("dense", 216, True),
+         ("dense", 225, False)]
+
+
+@pytest.mark.parametrize("kind,n,tables", MULTI)
+def test_batches(kind, n, tables):
+    """An instance beside one that differs by an entry of -1, which the product
+    kernel refuses: one shape class where both run that one's kernel."""
+    p = library()
+    D, F = instance(kind, n)
+    E = D.copy()
+    E[0, 1] = E[1, 0] = -1
+    S = 2
+    pairs = [(D, F), (E, F)]
+    qs = [p.Qap(*m) for m in pairs]
+    shape = p.pdit_launch_shape(qs[1], 1 << 20)
+    slots = shape["ctas"] * shape["replicas_per_cta"]
+    betas = [O.beta_schedule("linear", S, O.beta_max(*m)) for m in pairs]
+    for R, one in ((20, tables), (slots, False)):
+        items = [{"qap": q, "replicas": R, "sweeps": S, "beta": device(b), "seed": 4, "instance_id": k}
+                 for k, (q, b) in enumerate(zip(qs, betas))]
+        batch = p.Batch(items)
+        assert (batch.info()[0] == 1) == one
+        if R == 20:
+            batch.run()
+            for k, (o, m) in enumerate(zip([host(o) for o in batch.out], pairs)):
+                r = O.anneal(*m, betas[k], S, 4, 0, R, inst=k, threads=8)
+                assert int(o["best_cost"][0]) == r["cost"] and np.array_equal(o["best_perm"], r["perm"])
+        batch.close()
+    for q in qs:
+        q.close()
+
+
+def test_served():
+    """Few served replicas: slices on the kernels that batches take."""
+    p = library()
+    S, R = 9, 10
+    srv = p.Server(slice_sweeps=4, max_active=16)
+    insts = [instance(kind, n) for kind, n, _ in MULTI]
+    tickets = [srv.submit(D, F, R, S, 5, k) for k, (D, F) in enumerate(insts)]
+    while sum(srv.tick()):
+        pass
+    for k, (D, F) in enumerate(insts):
+        state, perm, cost, _ = srv.result(tickets[k])
+        r = O.anneal(D, F, O.beta_schedule("linear", S, O.beta_max(D, F)), S, 5, 0, R, inst=k, threads=8)
+        assert state == 2 and cost == r["cost"] and np.array_equal(perm, r["perm"])
+    srv.close()
