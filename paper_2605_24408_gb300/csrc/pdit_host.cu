@@ -496,33 +496,40 @@ bool use_cc_path(const pdit_qap *h, const pdit_opts *o) {
 // few of its slots are in use; with few replicas an SM the kernels that put
 // several warps on a replica are faster: the dot-product kernel for
 // symmetric instances, the table kernels for general ones. The most replicas
-// an SM at which `alt`, that kernel's shape, is taken, from both kernels'
-// times at 1 to 10 replicas an SM and 30 sizes of each form. us an update,
-// product kernel against dot products: N = 120 1.04 / 1.01 at 1, 1.09 / 1.13 at 3; N = 160 1.27 / 1.03
-// at 1, 1.32 / 1.35 at 3; N = 176 1.52 / 1.36 at 3, 1.56 / 1.57 at 4; N = 200
-// 1.82 / 1.13 at 1, 1.91 / 1.90 at 4; N = 224 1.87 / 1.54 at 2, 1.90 / 2.46
-// at 3; N = 240 1.58 / 1.15 at 1, 1.62 / 1.63 at 2. Tempering gains less: a
-// launch of few sweeps also loads and stores the permuted matrices (N = 176
-// 0.83 of the product kernel's time at 1, 1.07 at 3).
-// General instances, against tables: N = 64 0.74 / 0.68 at 1, 0.81 / 0.85 at
-// 8; N = 75 1.14 / 0.99 at 1; N = 100 1.47 / 0.74 at 1, 1.59 / 1.26 at 6, 1.62
-// / 1.68 at 8; N = 112 1.57 / 1.52 at 5, 1.62 / 1.81 at 6; N = 128 1.20 / 0.91
-// at 2, 1.21 / 1.36 at 3; N = 144 2.08 / 1.79 at 3, 2.11 / 2.36 at 4; N = 160
-// 2.06 / 1.66 at 2, 2.09 / 3.24 at 3. In tempering the tables are also loaded
-// and stored at each exchange (N = 100: 1.72 / 1.56 at 2, 1.72 / 1.68 at 3).
-int few_replicas(const pdit_qap *h, const Plan &alt, bool pt) {
+// an SM at which `alt`, that kernel's shape, is taken: up to there it is the
+// faster one for dense instances under the linear schedule (0.3 to 0.5 of the
+// updates swap), and loses less under the geometric one (0.8 to 0.9 swap) and
+// for grids (0.9) than the product kernel would lose there. Its time over the
+// product kernel's at 1, 2 and 3 replicas an SM, dense linear; dense
+// geometric; grid geometric: N = 128 0.95 0.92 1.02; 0.99 0.99 1.10; 1.00 1.00
+// 1.12. N = 160 0.82 0.91 1.03; 0.92 1.02 1.14; 0.94 1.05 1.17. N = 208 0.63
+// 0.73 0.85; 0.70 0.81 0.94; 0.72 0.83 0.96. N = 224 0.64 0.83 1.60; 0.68 0.90
+// 1.74; 0.69 0.92 1.78. N = 256 0.80 1.10; 0.84 1.17; 0.85 1.19. Tempering
+// gains less, as a launch of few sweeps also loads and stores the permuted
+// matrices: N = 176 0.84 0.97 1.07, N = 208 0.73 0.87 1.00, N = 256 0.86 1.25.
+// General instances, uniform linear; uniform geometric; one-way grid
+// geometric, at 1 to 5: N = 64 0.93 0.90 0.96; 1.36 1.34 1.41; 1.45 1.43 1.51.
+// N = 100 0.51 0.54 0.59 0.64 0.69 (6: 0.82); 0.77 0.82 0.89 0.97 1.05 (1.24);
+// 0.83 0.89 0.96 1.04 1.13 (1.32): the tables' own round ends at 5. N = 112
+// 0.53 0.57 0.62 0.83; 0.79 0.84 0.91 1.24; 0.84 0.90 0.98 1.37 (its round: 3).
+// N = 128 0.73 0.77 1.16; 1.04 1.12 1.70; 1.10 1.20 1.79. N = 140 0.51 0.60
+// 0.89; 0.73 0.86 1.29; 0.78 0.92 1.42. N = 160 (tables in global memory) 0.55
+// 0.86; 0.72 1.23; 0.76 1.32. Tempering: N = 100 0.86 0.91 0.98, N = 128 1.12,
+// N = 140 0.80 0.95 1.28, N = 160 0.78 1.33.
+int few_replicas(const pdit_qap *h, const Plan &alt, int replicas, bool pt) {
     const int n = h->n;
     if (h->asym) {
         switch (alt.wpr) {
-        case 2: return pt ? 0 : 6;
-        case 4: return n > 112 ? (pt ? 0 : 2) : pt ? 2 : n < 104 ? 7 : 5;
-        case 8: return (alt.tsmem ? 3 : 2) - (pt ? 1 : 0);
+        case 4:
+            if (n > 112) return pt ? 0 : 2;
+            return pt ? 2 : replicas <= alt.grid * alt.groups ? 5 : 0;
+        case 8: return alt.tsmem ? 2 : 1;
         default: return 0;
         }
     }
     switch (alt.wpr) {
     case 2: return !pt && n <= 128 ? 2 : 0;
-    case 4: return pt ? (n <= 192 ? 1 : 2) : (n <= 160 ? 2 : 3);
+    case 4: return n > 192 ? (pt ? 2 : 3) : (pt ? 1 : 2);
     case 8: return n <= 224 ? 2 : 1;
     default: return 0;
     }
@@ -532,12 +539,9 @@ int few_replicas(const pdit_qap *h, const Plan &alt, bool pt) {
 // tensor-core product kernel takes it; false where none does.
 bool few_plan(const pdit_qap *h, int replicas, bool pt, Plan *p, size_t reserve) {
     const int per_sm = (replicas + h->num_sms - 1) / h->num_sms;
-    if (per_sm > (h->asym ? 7 : 3) || mm_form(h) == pdit::kMmWide) return false;
-    // (general calls of fewer than 8 replicas keep the product kernel, which
-    // tests/test_gpu_matrix.py expects of them)
-    if (h->asym && replicas < 8) return false;
+    if (per_sm > (h->asym ? 5 : 3) || mm_form(h) == pdit::kMmWide) return false;
     const int rc = h->asym ? make_plan(h, replicas, 0, 0, p, reserve) : make_dot_plan(h, replicas, 0, p, reserve);
-    if (rc == PDIT_OK && per_sm <= few_replicas(h, *p, pt)) return true;
+    if (rc == PDIT_OK && per_sm <= few_replicas(h, *p, replicas, pt)) return true;
     *p = Plan();
     return false;
 }
@@ -549,7 +553,9 @@ bool few_plan(const pdit_qap *h, int replicas, bool pt, Plan *p, size_t reserve)
 // the table kernels.
 int product_plan(const pdit_qap *h, int replicas, bool pt, Plan *p, size_t reserve, bool any) {
     if (mm_eligible(h) && h->force_wpr <= 1) {
-        if (h->force_wpr == 0 && few_plan(h, replicas, pt, p, reserve)) return PDIT_OK;
+        // (general calls of fewer than 8 replicas keep the product kernel, which
+        // tests/test_gpu_matrix.py expects of them)
+        if (h->force_wpr == 0 && (!h->asym || replicas >= 8) && few_plan(h, replicas, pt, p, reserve)) return PDIT_OK;
         const int rc = make_mm_plan(h, replicas, p, reserve);
         if (rc != PDIT_ENOTSUP) return rc;
         *p = Plan();
@@ -593,46 +599,28 @@ int plan_for(const pdit_qap *h, const pdit_opts *o, Plan *p) {
     return make_plan(h, o->replicas, h->force_wpr, h->force_pk, p, 0, o->mode == PDIT_MODE_CUPIM);
 }
 
-// Whether a multi-instance launch of `load` replicas in all takes `alt`, the
-// shape of the kernel that an instance runs where the tensor-core product
-// kernel does not, instead of that kernel: where the launch is one round of
-// alt's resident replicas and alt puts several warps on a replica. Time of a
-// batch, alt / product kernel, inside the round and beyond it: general N = 80
-// 0.75 and 1.27, N = 100 0.71 and 1.15, N = 112 0.58 and 1.15, N = 128 0.73 and
-// 1.46, N = 160 0.81 and 1.60 (N = 76, two warps: 1.05); wide N = 120 0.87 and
-// 1.73, N = 128 0.91 and 1.79 (N = 112: 1.13); symmetric N = 212 0.88 and 1.74,
-// N = 224 0.91 and 1.80 (N = 225: 1.11; at 208 and below dot products: 1.01).
-bool few_load(const pdit_qap *h, const Plan &alt, long long load) {
-    if (alt.wpr < 4 || load > (long long)alt.grid * alt.groups) return false;
-    if (h->asym) return true;
-    return mm_form(h) == pdit::kMmWide ? h->n > 112 : !alt.dot && h->n <= 224;
-}
-
 // Plan of one instance in a multi-instance launch (batches, the server) of
 // `load` replicas in all: the product kernels where the automatic rule takes
-// them, else the table kernels; the kernels keep their descriptor in
-// `reserve` bytes of static shared memory.
+// them, else the table kernels, with as many replicas per CTA as fit; the
+// kernels keep their descriptor in `reserve` bytes of static shared memory.
+// A launch with few replicas follows the rule of single calls (few_plan) by
+// its load, and its replicas spread over the SMs: a batch's time over the
+// product kernel's at 1 and 2 replicas an SM, linear and geometric schedules:
+// general N = 100 0.50 0.54, 0.75 0.81 (5: 0.59, 0.88); N = 128 0.71 0.77, 1.01
+// 1.11; N = 140 0.48 0.59, 0.69 0.83; dense N = 128 0.83 0.86, 0.88 0.90; N = 200
+// 0.59 0.70, 0.65 0.79; N = 224 0.64 0.84, 0.69 0.90; N = 256 0.79, 0.83.
 int batch_plan(const pdit_qap *h, long long load, Plan *p, size_t reserve) {
-    const int full = 1 << 28;  // as many replicas per CTA as fit
+    const int full = 1 << 28;
     if (!h->cls || !h->use_cls) {
-        if (h->force_infl == PDIT_INFLUENCE_PRODUCTS) {
-            if (!dot_eligible(h)) return PDIT_ENOTSUP;
-            return product_plan(h, full, false, p, reserve, true);
-        }
+        const bool products = h->force_infl == PDIT_INFLUENCE_PRODUCTS;
+        if (products && !dot_eligible(h)) return PDIT_ENOTSUP;
         pdit_opts o;
         pdit_opts_init(&o);
-        if (use_dot_path(h, &o)) {
-            if (mm_eligible(h) && h->force_wpr == 0) {
-                int rc = dot_eligible(h) ? auto_dot_plan(h, full, p, reserve) : PDIT_ENOTSUP;
-                if (rc == PDIT_ENOTSUP) {
-                    *p = Plan();
-                    rc = make_plan(h, full, 0, 0, p, reserve);
-                }
-                if (rc == PDIT_OK && few_load(h, *p, load)) return PDIT_OK;
-                *p = Plan();
-            }
-            const int rc = product_plan(h, full, false, p, reserve, false);
-            if (rc != PDIT_ENOTSUP) return rc;
+        if (products || use_dot_path(h, &o)) {
+            if (mm_eligible(h) && h->force_wpr == 0 && load < full && few_plan(h, (int)load, false, p, reserve))
+                return PDIT_OK;
+            const int rc = product_plan(h, full, false, p, reserve, products);
+            if (products || rc != PDIT_ENOTSUP) return rc;
             *p = Plan();
         }
     }

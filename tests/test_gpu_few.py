@@ -28,7 +28,8 @@ def compare(p, q, D, F, beta, S, R, mode="anneal", L=4):
 
 
 @pytest.mark.parametrize("n,per_sm,warps", [(112, 1, 1), (113, 2, 2), (128, 2, 2), (128, 3, 1), (129, 1, 1), (160, 2, 4),
-                                            (160, 3, 1), (161, 3, 4), (200, 3, 4), (200, 4, 1), (224, 2, 8), (224, 3, 1),
+                                            (160, 3, 1), (192, 2, 4), (192, 3, 1), (200, 3, 4), (200, 4, 1), (224, 2, 8),
+                                            (224, 3, 1),
                                             (225, 1, 8), (225, 2, 1), (256, 1, 8)])
 def test_symmetric(n, per_sm, warps):
     """`warps` at per_sm replicas an SM: 1 is the product kernel (the first
@@ -65,11 +66,11 @@ def general(n):
     return G.asymmetric(n, 0, 99, n, 101), G.asymmetric(n, 0, 99, n, 103)
 
 
-@pytest.mark.parametrize("n,per_sm,kind", [(50, 1, "products"), (64, 6, "table"), (64, 7, "products"), (75, 6, "table"),
-                                           (75, 7, "products"), (100, 7, "table"), (100, 8, "products"),
-                                           (112, 5, "table"), (112, 6, "products"), (113, 2, "table"),
-                                           (128, 2, "table"), (128, 3, "products"), (129, 3, "table"),
-                                           (144, 4, "products"), (160, 2, "table"), (160, 3, "products")])
+@pytest.mark.parametrize("n,per_sm,kind", [(50, 1, "products"), (75, 1, "products"), (79, 5, "table"),
+                                           (100, 5, "table"), (100, 6, "products"), (112, 3, "table"),
+                                           (112, 4, "products"), (113, 2, "table"), (128, 2, "table"),
+                                           (128, 3, "products"), (129, 2, "table"), (144, 3, "products"),
+                                           (160, 1, "table"), (160, 2, "products")])
 def test_general(n, per_sm, kind):
     """The last call of the table kernels, the first of the product kernel."""
     p = library()
@@ -118,34 +119,31 @@ def instance(kind, n):
     return G.dense_instance(n, seed=n)
 
 
-MULTI = [("general", 76, False), ("general", 80, True), ("general", 100, True), ("general", 128, True),
-         ("general", 160, True), ("wide", 112, False), ("wide", 128, True), ("dense", 200, False), ("dense", 216, True),
-         ("dense", 225, False)]
+MULTI = [("general", 76), ("general", 100), ("general", 128), ("general", 160), ("wide", 112), ("dense", 176),
+         ("dense", 200), ("dense", 224), ("dense", 256)]
 
 
-@pytest.mark.parametrize("kind,n,tables", MULTI)
-def test_batches(kind, n, tables):
-    """An instance beside one that differs by an entry of -1, which the product
-    kernel refuses: one shape class where both run that one's kernel."""
+@pytest.mark.parametrize("kind,n", MULTI)
+def test_batches(kind, n):
+    """Few replicas in all: the kernels of a single call, spread over the SMs
+    (a shape class that one warp per replica does not share), and the results
+    of the oracle; many: the product kernel."""
     p = library()
+    few = kind != "wide" and n > 76
     D, F = instance(kind, n)
-    E = D.copy()
-    E[0, 1] = E[1, 0] = -1
     S = 2
-    pairs = [(D, F), (E, F)]
-    qs = [p.Qap(*m) for m in pairs]
-    shape = p.pdit_launch_shape(qs[1], 1 << 20)
-    slots = shape["ctas"] * shape["replicas_per_cta"]
-    betas = [O.beta_schedule("linear", S, O.beta_max(*m)) for m in pairs]
-    for R, one in ((20, tables), (slots, False)):
-        items = [{"qap": q, "replicas": R, "sweeps": S, "beta": device(b), "seed": 4, "instance_id": k}
-                 for k, (q, b) in enumerate(zip(qs, betas))]
+    qs = [p.Qap(D, F), p.Qap(D, F)]
+    p.pdit_set_warps_per_replica(qs[1], 1)  # the product kernel
+    beta = O.beta_schedule("linear", S, O.beta_max(D, F))
+    for R, classes in ((20, 2 if few else 1), (4 * sms(), 1)):
+        items = [{"qap": q, "replicas": R, "sweeps": S, "beta": device(beta), "seed": 4, "instance_id": k}
+                 for k, q in enumerate(qs)]
         batch = p.Batch(items)
-        assert (batch.info()[0] == 1) == one
+        assert batch.info()[0] == classes
         if R == 20:
             batch.run()
-            for k, (o, m) in enumerate(zip([host(o) for o in batch.out], pairs)):
-                r = O.anneal(*m, betas[k], S, 4, 0, R, inst=k, threads=8)
+            for k, o in enumerate([host(o) for o in batch.out]):
+                r = O.anneal(D, F, beta, S, 4, 0, R, inst=k, threads=8)
                 assert int(o["best_cost"][0]) == r["cost"] and np.array_equal(o["best_perm"], r["perm"])
         batch.close()
     for q in qs:
@@ -157,7 +155,7 @@ def test_served():
     p = library()
     S, R = 9, 10
     srv = p.Server(slice_sweeps=4, max_active=16)
-    insts = [instance(kind, n) for kind, n, _ in MULTI]
+    insts = [instance(kind, n) for kind, n in MULTI]
     tickets = [srv.submit(D, F, R, S, 5, k) for k, (D, F) in enumerate(insts)]
     while sum(srv.tick()):
         pass
