@@ -1740,14 +1740,43 @@ std::vector<int> unit_groups(const std::vector<UnitLoad> &loads, int num_sms) {
     double total = 0.0;
     for (const UnitLoad &u : loads)
         if (u.plan->mm) total += unit_cost(u) * u.replicas / 16.0 * (u.plan->lanes == 16 ? 0.5 : 1.0) / num_sms;
+    // Halve the units of the instances that outlast it, all together. Halves
+    // that no longer fit one round of the resident CTAs wait for the first to
+    // end, about a short unit beyond the evenly spread time: where that takes
+    // well longer than the round did (an estimate, so by a quarter), the launch
+    // stays one round (general N = 120, 800 replicas: 200 units of 4 on 152 SMs
+    // would be two; 0.55 of their time).
+    struct Time {
+        double rounds = 0.0, spread = 0.0, longest = 0.0, shortest = 1e300;
+    };
+    auto time_of = [&](const std::vector<int> &k) {
+        Time t;
+        for (size_t q = 0; q < loads.size(); ++q) {
+            const UnitLoad &u = loads[q];
+            if (!u.plan->mm) continue;
+            const double share = (double)((u.replicas + k[q] - 1) / k[q]) / u.plan->grid;
+            const double cost = unit_cost(u) * (0.55 + 0.45 * k[q] / 16.0);
+            t.rounds += share;
+            t.spread += share * cost;
+            t.longest = std::max(t.longest, cost);
+            t.shortest = std::min(t.shortest, cost);
+        }
+        return t;
+    };
     std::vector<int> g;
-    for (const UnitLoad &u : loads) {
-        int k = u.plan->groups;
-        if (u.plan->mm)
-            while (k > 4 && unit_cost(u) * (0.55 + 0.45 * k / 16.0) > total) k = (k + 1) / 2;
-        g.push_back(k);
+    for (const UnitLoad &u : loads) g.push_back(u.plan->groups);
+    for (;;) {
+        std::vector<int> half = g;
+        for (size_t q = 0; q < loads.size(); ++q)
+            if (loads[q].plan->mm && g[q] > 4 && unit_cost(loads[q]) * (0.55 + 0.45 * g[q] / 16.0) > total)
+                half[q] = (g[q] + 1) / 2;
+        if (half == g) return g;
+        const Time now = time_of(g), next = time_of(half);
+        if (now.rounds <= 1.0 && next.rounds > 1.0 &&
+            std::max(next.longest, next.spread + next.shortest) > 1.25 * now.longest)
+            return g;
+        g = half;
     }
-    return g;
 }
 
 // Per instance: reset its time-to-target outputs and stop flag.

@@ -164,3 +164,23 @@ def test_served():
         r = O.anneal(D, F, O.beta_schedule("linear", S, O.beta_max(D, F)), S, 5, 0, R, inst=k, threads=8)
         assert state == 2 and cost == r["cost"] and np.array_equal(perm, r["perm"])
     srv.close()
+
+
+@pytest.mark.parametrize("n,R", [(120, 5), (128, 8)])
+def test_batch_units_of_one_round(n, R):
+    """Loads where units of 4 replicas would no longer fit the SMs at once:
+    the batch equals single calls."""
+    p = library()
+    D, F = general(n)
+    R *= sms()
+    S = 2
+    with p.Qap(D, F) as q:
+        db = device(O.beta_schedule("linear", S, O.beta_max(D, F)))
+        items = [{"qap": q, "replicas": R // 2 + k, "sweeps": S, "beta": db, "seed": 4, "instance_id": k}
+                 for k in range(2)]
+        batch = p.Batch(items)
+        batch.run()
+        for k, o in enumerate([host(o) for o in batch.out]):
+            g = host(p.anneal_device(q, R // 2 + k, db, S, 4, instance_id=k))
+            assert int(o["best_cost"][0]) == int(g["best_cost"][0]) and np.array_equal(o["best_perm"], g["best_perm"])
+        batch.close()
