@@ -459,11 +459,12 @@ int make_small_plan(const pdit_qap *h, int replicas, Plan *p) {
 }
 
 // Whether a call runs the small kernel: at most 32 locations, symmetric, a
-// sequential mode, no table dump, and no setting that asks for another kernel
-// (dot products, pending terms, more than one warp per replica).
+// sequential mode, no table dump, no setting that asks for another kernel or
+// shapes the table kernels (influence, pending terms, placement) and no more
+// than one warp per replica asked for.
 bool use_small_path(const pdit_qap *h, const pdit_opts *o) {
     return h->n <= 32 && !h->asym && o->mode != PDIT_MODE_CUPIM && !o->tables && h->force_wpr <= 1 &&
-           h->force_pk <= 1 && h->force_place != PDIT_PLACE_GLOBAL && h->force_infl != PDIT_INFLUENCE_PRODUCTS;
+           h->force_pk == 0 && h->force_place == PDIT_PLACE_AUTO && h->force_infl == PDIT_INFLUENCE_AUTO;
 }
 
 // Launch shape of the concurrent-update kernel: one CTA per replica.
