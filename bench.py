@@ -905,7 +905,7 @@ def main():
         macs = (1 if -(-n // 16) == 7 else 2) * (16 * -(-n // 16)) ** 2
         alu = {"op": "mma.sync f16 multiply-add", "per_update": macs, "achieved_ops_per_s": macs * upd_rank / kernel_s,
                "peak_key": "mma_f16_macs_per_clk_sm"}
-    elif products and form is not None and not args.wpr:
+    elif products and form is not None and shape["warps_per_replica"] == 1:
         # no table: the kernel's own traffic is the figure
         bpu = bpu_design = mm_bytes_per_update(n, accept_frac, form)
         basis = "the tensor-core product kernel's own shared-memory traffic (mm_bytes_per_update, %s form)" % form
@@ -922,8 +922,8 @@ def main():
         dp4a = product_dp4a_per_update(n)
         alu = {"op": "dp4a", "per_update": dp4a, "achieved_ops_per_s": dp4a * upd_rank / kernel_s,
                "peak_key": "dp4a_ops_per_clk_sm"}
-    elif not general and n <= 32 and shape["pending_swaps"] == 1 and shape["warps_per_replica"] == 1 and \
-            args.mode != "cupim":
+    elif not general and n <= 32 and args.wpr <= 1 and not (args.pk or args.place) and \
+            infl == P.PDIT_INFLUENCE_AUTO and args.mode != "cupim":
         # the table's row in registers and a copy in shared memory: the
         # method's traffic, of which the kernel moves a part
         kname = "small_kernel<%d>" % (16 if n <= 16 else 24 if n <= 24 else 32)
