@@ -67,10 +67,10 @@ extern "C" {
 /* Device status bits (opts.status). */
 #define PDIT_STATUS_ENERGY_AUDIT 1 /* tracked energy != energy recomputed (from the table or
                                       the flow-class vector at a resume or at the end; from
-                                      Eq. 1 at the end of every dot-kernel call) */
+                                      Eq. 1 at the end of every call of the other kernels) */
 #define PDIT_STATUS_SCHEDULE 2     /* a part of a replica's sweeps waited past its bound for the
-                                      part before it (dot kernel, more replicas than resident
-                                      slots); the call stopped early and its results are not valid */
+                                      part before it (calls in parts, see pdit_workspace_bytes);
+                                      the call stopped early and its results are not valid */
 
 typedef struct pdit_qap pdit_qap;
 
@@ -107,17 +107,19 @@ int pdit_set_warps_per_replica(pdit_qap *h, int wpr);
 
 /*
  * pdit_autotune -- time every compiled thread mapping (warps per replica) of
- * the dot-product kernel (eligible instances; see pdit_set_influence) and of
- * the table kernels, with their table-update batching (1, 4 or 16 pending
- * terms), the table placement (shared or global memory, when both are
- * possible) and, where the tables live in global memory, replicas per CTA
- * (1..4 besides the built-in choice) valid for this instance on a short run
- * of `replicas` chains over the DEVICE schedule beta[sweeps] (CUDA events on
- * the handle's stream), keep the fastest for later calls on this handle and
- * write it to shape[0] (warps per replica) and shape[1] (pending terms; 1 for
- * the dot kernel) when shape is not NULL (pdit_launch_shape reports the
- * replicas per CTA and which kernel). Synchronous; allocates and frees
- * small temporary buffers. Results of later calls do not depend on the
+ * the product kernels (symmetric byte-valued instances; see
+ * pdit_set_influence) and of the table kernels, with their table-update
+ * batching (1, 4 or 16 pending terms), the table placement (shared or global
+ * memory, when both are possible) and, where the tables live in global
+ * memory, replicas per CTA (1..4 besides the built-in choice), and the
+ * built-in choice where no setting asks for its kernel (the small kernel, the
+ * product kernel's wide and general forms), those valid for this instance, on
+ * a short run of `replicas` chains over the DEVICE schedule beta[sweeps] (CUDA
+ * events on the handle's stream), keep the fastest for later calls on this
+ * handle and write it to shape[0] (warps per replica) and shape[1] (pending
+ * terms; 1 for kernels without) when shape is not NULL (pdit_launch_shape
+ * reports the replicas per CTA and which kernel). Synchronous; allocates and
+ * frees small temporary buffers. Results of later calls do not depend on the
  * choice. Errors: PDIT_EINVAL, PDIT_ENOTSUP, PDIT_ECUDA.
  */
 int pdit_autotune(pdit_qap *h, int replicas, const float *beta, int sweeps, int *shape);
@@ -161,7 +163,7 @@ int pdit_launch_shape(const pdit_qap *h, int replicas, int *shape);
 /* Influence entries (pdit_set_influence). */
 #define PDIT_INFLUENCE_AUTO 0     /* products where eligible and no table knob is set, else the table */
 #define PDIT_INFLUENCE_TABLE 1    /* the influence table of Eq. 2, updated after every accepted swap */
-#define PDIT_INFLUENCE_PRODUCTS 2 /* dot products of byte rows of D and of the permuted F (no table) */
+#define PDIT_INFLUENCE_PRODUCTS 2 /* products of byte rows of D and F, or of the permuted F (no table) */
 
 /*
  * pdit_set_influence -- how later sequential-mode calls on this handle obtain
@@ -184,7 +186,9 @@ int pdit_launch_shape(const pdit_qap *h, int replicas, int *shape);
  *                             next call). Above 32 locations, zero diagonals
  *                             and entries in 0..127 form the products of many
  *                             replicas on the tensor cores, from D and F
- *                             themselves and no matrix per replica. Two-level-flow instances keep the
+ *                             themselves and no matrix per replica (with few
+ *                             replicas an SM above 112 locations: the dot
+ *                             products). Two-level-flow instances keep the
  *                             flow-class kernel unless pdit_set_class_update
  *                             turns it off.
  *   PDIT_INFLUENCE_AUTO     : unless a table knob (pending swaps,
@@ -194,7 +198,10 @@ int pdit_launch_shape(const pdit_qap *h, int replicas, int *shape);
  *                             (symmetric with entries to 127, or to 2047 at
  *                             128 locations at most; general with entries to
  *                             127 and 8 (N + 2) max D max F below 2^24, to
- *                             160 locations); symmetric instances of at most
+ *                             160 locations; with few replicas an SM, a
+ *                             kernel of several warps a replica: dot
+ *                             products, for general instances the table);
+ *                             symmetric instances of at most
  *                             32 locations, tables in registers; in the
  *                             concurrent-update mode, one tensor-core
  *                             product per iteration (symmetric, zero
@@ -324,18 +331,18 @@ void pdit_opts_init(pdit_opts *o);
  * which selects the table kernels): query it with the options of the call.
  * Returns 0 for invalid input.
  * The workspace holds every replica's state between calls (permutation,
- * energy, best-so-far, counters, and in PT mode the influence tables), so a
- * call with PDIT_FLAG_RESUME continues exactly where the previous one
- * stopped. With more replicas than the GPU holds at once (not a whole
- * number of rounds), the dot-product kernel and the table kernels with
- * tables in shared memory run each replica's sweeps as parts, separate work
- * units of one launch, in every mode. The parts are up to 16 of 8 to 1000
- * sweeps, or of one sweep per PT exchange period. The workspace then also
- * holds every replica's table (the dot kernel's permuted flow matrix, about
- * n * n bytes; an n x stride int32 influence table) and a 4-byte part
- * counter, whatever the sweep range, so a resumed call over a longer range
- * fits the workspace of the call before it. Results do not depend on the
- * parts.
+ * energy, best-so-far, counters, and in PT mode the influence tables of the
+ * table and dot-product kernels), so a call with PDIT_FLAG_RESUME continues
+ * exactly where the previous one stopped. With more replicas than the GPU
+ * holds at once (not a whole number of rounds), every kernel but the
+ * flow-class kernel and tables in global memory runs each replica's sweeps as
+ * parts, separate work units of one launch, in every mode. The parts are up to
+ * 16 of 8 to 1000 sweeps, or of one sweep per PT exchange period. The
+ * workspace then also holds a 4-byte part counter for every replica and, for
+ * the table and dot-product kernels, its table (the dot kernel's permuted flow
+ * matrix, about n * n bytes; an n x stride int32 influence table), whatever the
+ * sweep range, so a resumed call over a longer range fits the workspace of the
+ * call before it. Results do not depend on the parts.
  */
 size_t pdit_workspace_bytes(const pdit_qap *h, const pdit_opts *o);
 

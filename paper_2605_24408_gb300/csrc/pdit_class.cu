@@ -22,9 +22,10 @@
 // memory keeps the copies other threads read (G_i, and the facilities for
 // swaps).
 //
-// Bound: issue slots (about 190 instructions an update at N = 256 and one
-// warp per replica); 27 one-warp replicas an SM of 64 registers a thread hide
-// the chain, and 4096 replicas are one round.
+// Bound: issue slots (352 warp instructions an update at N = 256 and one warp
+// per replica; issue 75% busy); 27 one-warp replicas an SM of 72 registers a
+// thread (66 bytes of spill stores, 96 of loads) hide the chain, and 4096
+// replicas are one round.
 #include "pdit_sweep.cuh"
 
 namespace pdit {

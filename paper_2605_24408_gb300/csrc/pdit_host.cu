@@ -574,8 +574,8 @@ bool use_dot_path(const pdit_qap *h, const pdit_opts *o) {
     return h->force_infl == PDIT_INFLUENCE_AUTO && h->force_pk == 0 && h->force_place == PDIT_PLACE_AUTO;
 }
 
-// Launch plan of a call: the flow-class kernel, the dot-product kernel or
-// the table kernels.
+// Launch plan of a call: the flow-class kernel, the concurrent kernel, the
+// small kernel, a product kernel or the table kernels.
 int plan_for(const pdit_qap *h, const pdit_opts *o, Plan *p) {
     if (use_class_path(h, o)) return make_class_plan(h, o->replicas, h->force_wpr, p);
     if (use_cc_path(h, o)) {
@@ -634,8 +634,7 @@ struct Workspace {
     size_t bytes;
 };
 
-// Parts a launch of `span` sweeps of the dot or table kernels splits every
-// replica's sweeps into. With more replicas than resident slots, whole units
+// Parts a launch of `span` sweeps splits every replica's sweeps into. With more replicas than resident slots, whole units
 // leave the last round's idle slots idle until it ends (at n100, 4096
 // replicas in 2432 slots ran at 0.85 of the full-round rate; the general
 // form's table kernel, 4096 in 760 slots, at 0.94); parts run as separate
@@ -645,8 +644,8 @@ struct Workspace {
 // the replicas fill whole rounds, for the flow-class kernel and for tables
 // in global memory.
 // Whether launches of the plan may be split (the replicas exceed the slots
-// and are not a whole number of rounds; dot kernel or tables in shared
-// memory). It does not depend on the sweep range, so neither does the
+// and are not a whole number of rounds; not the flow-class kernel or tables in
+// global memory). It does not depend on the sweep range, so neither does the
 // workspace: a resumed call over a longer range fits the workspace of the
 // call before it.
 bool may_split(const pdit_opts *o, const Plan &p) {
@@ -1337,8 +1336,8 @@ int pdit_autotune(pdit_qap *h, int replicas, const float *beta, int sweeps, int 
     // the built-in choice plus 1..4 where the tables live in global memory
     // (there the built-in choice is an L2-capacity estimate). The flow-class
     // kernel keeps no table: only its warps per replica vary.
-    // The dot-product kernel (eligible instances, unless the caller fixed the
-    // table) adds its compiled warps-per-replica shapes.
+    // The product kernels (eligible instances, unless the caller fixed the
+    // table) add their compiled warps-per-replica shapes.
     std::vector<Knobs> cand;
     const int cover = cover_for(h->n);
     const int tbl = cls ? keep.infl : (int)PDIT_INFLUENCE_TABLE;

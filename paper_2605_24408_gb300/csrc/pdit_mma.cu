@@ -40,8 +40,12 @@
 // 64 replicas, 1.6 (N = 33) to 6.6 (N = 112) with 4096.
 //
 // Bound: the latency of an update's chain of about 450 instructions a warp
-// (issue slots 45% busy, 15 warps an SM at the register limit; shared-memory
-// pipe 67%, tensor pipe 26%). Byte permutes that form a gather's address from
+// (N = 100: issue slots 45% busy, shared-memory pipe 67%, tensor pipe 26%).
+// The launch bound of two CTAs an SM holds 16 lanes at 16 warps an SM; at 97
+// to 128 locations registers do (128 a thread; the spills are 36 / 64 bytes of
+// stores / loads at 97, 94 / 196 at 113 locations, 150 / 304 in the wide form),
+// below 81 fewer would do. With few replicas an SM other kernels are faster
+// (few_replicas in pdit_host.cu). Byte permutes that form a gather's address from
 // its row's, warp-uniform control and replicas paired in warps from the first
 // took N = 100, 4096 replicas, from 2.13e9 to 2.39e9 updates/s (1.12e9 with
 // the dot-product kernel); N = 256, 2048 replicas: 7.3e8 (1.6e8 with the table
@@ -63,7 +67,6 @@ struct MmShape {
     static constexpr bool ASYM = FORM == kMmGeneral, WIDE = FORM == kMmWide;
     using V = typename std::conditional<WIDE, int, float>::type;      // energies and influence entries
     using E = typename std::conditional<WIDE, long long, int>::type;  // energies of states
-    static constexpr int ES = WIDE ? 2 : 1;       // bytes of a table entry
     static constexpr int NP = K * LPR;            // padded size
     static constexpr int MT = NP / 16;            // 16-row tiles of D and of F; 16-deep steps of a product
     static constexpr int NW = LPR == 16 ? 8 : 16; // warps per CTA

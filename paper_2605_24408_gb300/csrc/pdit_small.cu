@@ -19,12 +19,12 @@
 // (8 (n + 2) max|D| max|F| < 2^24: exact, and two products per instruction),
 // else int32.
 //
-// Bound: the latency of the chain, 600 clocks an update at N = 12 (64
-// replicas, 0.42 of the updates swap) and 780 at N = 30 (0.84 swap), against
-// 1070 and 1400 with the dot-product kernel; one warp alone issues about one
-// instruction in three clocks. N = 30, 1024 replicas, 5000 sweeps: 62 ms (125
+// Bound: the latency of the chain, 560 clocks an update at N = 12 (64
+// replicas, 0.42 of the updates swap) and 850 at N = 30 (0.84 swap), against
+// 1070 and 1700 with the dot-product kernel; one warp alone issues about one
+// instruction in three clocks. N = 30, 1024 replicas, 5000 sweeps: 61.4 ms (125
 // ms with the dot-product kernel, 72 ms with the table changed in the swap
-// itself).
+// itself). The row's copy is stored in every update, changed or not.
 #include <type_traits>
 
 #include "pdit_sweep.cuh"

@@ -69,7 +69,7 @@ struct SweepArgs {
     int fresh;             // start from a Fisher-Yates permutation
     int table_in;          // take the influence table from `tables` instead of rebuilding it
     int table_out;         // leave the influence table in `tables` at the end
-    int audit;             // tensor-core product kernel: check the final energies against Eq. 1
+    int audit;             // tensor-core product kernel: the call's last launch, which checks its energies against Eq. 1
     // per-replica state, indexed by local replica id
     int32_t *perm;
     int32_t *best_perm;
@@ -105,7 +105,7 @@ struct SweepArgs {
 struct GroupScratch {
     unsigned long long wtot[8];
     int wmin[8];
-    int sel_jf, sel_d;  // the drawn outcome: location | facility << 16, energy change
+    int sel_jf, sel_d;  // the drawn outcome: location | facility << 8 | tag << 16, energy change
     int part_end;       // dot kernel: the last sweep (exclusive) of the part being run
     int item;
     int stop;
