@@ -43,10 +43,12 @@ struct CcShape {
     static constexpr int GS = 16 * (MT | 1);  // row stride of D and G, bytes
     static constexpr int FS = 256;            // of F: an entry's address is its row's with the column for the low byte
     static constexpr int CTAS = (MT >= 7 ? 512 : MT >= 5 ? 640 : 768) / T;  // resident CTAs an SM aimed at (more spill)
-    // S = J + J^T, J = D G exchanged through shared memory, where that takes
-    // no CTA away; else both products. 4096 replicas x 60 iterations, J or
-    // both: N = 100 7.0 or 7.8 ms; N = 96 5.8 or 5.2, N = 64 2.2 or 2.0 (J's
-    // memory leaves fewer CTAs an SM); N = 128: J leaves one.
+    // S = J + J^T, J = D G exchanged through shared memory, at 97 to 112
+    // locations, where it is faster; else both products. 4096 replicas x 60
+    // iterations, J or both: N = 100 7.0 or 7.8 ms; N = 96 5.8 or 5.2, N = 64
+    // 2.2 or 2.0 (J's memory leaves fewer CTAs an SM); N = 128: J leaves one;
+    // N = 32 0.64 or 0.61, N = 16 0.32 or 0.31 (as many CTAs, but the products
+    // are short and the exchange is not).
     static constexpr bool TR = MT == 7;
     static constexpr int CS = NP + 4;  // row stride of J, floats: the transposed reads of a warp in distinct banks (NP = 112)
     // shared memory, bytes (F first: its rows are 256-byte aligned)
